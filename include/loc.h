@@ -96,20 +96,18 @@ typedef struct {
 } loc_params;
 
 #define LOC_TILE_CONFIGS 18    /* tile rows x 64 columns, threads: 1: 32 (256), 2: 16 (256),
-                                  3: 16 (128), 4: 16 (512), 5: 32 (512); warp-specialised
+                                  4: 16 (512), 5: 32 (512); the streaming kernel, one
+                                  persistent CTA per SM: 3 and 17: 28 (512), 16: the same with
+                                  the argmax combined in the step; warp-specialised
                                   producer/consumer pipelines: 6: 16 (256), 7: 8 (256),
                                   13: 14 (256); with cells paired 32 columns apart on the
                                   packed FP32 pipe: 8: 16 (128), 9: 16 (256), 10: 32 (256),
                                   11: 8 (128), 12: 16 (128, 2 raw stages); warp-specialised
                                   with the producers split into S-pass and X-pass warps:
-                                  14: 16 (320), 15: 14 (288), 16: 28 (512, one CTA per SM);
-                                  3 and 2 as a software pipeline over the planes (one CTA
-                                  barrier per plane): 17: 16 (128), 18: 16 (256).
+                                  14: 16 (320), 15: 14 (288); 2 as a software pipeline over
+                                  the planes (one CTA barrier per plane): 18: 16 (256).
                                   With tile = 0 a grid of at least 8 sixteen-row tiles per SM
-                                  takes 17 (FP32) or 3 (16-bit storage); smaller grids take
-                                  whichever of 6, 15 and 16 gives
-                                  the busiest SM the fewest rows to blur (tile rows + 4 per
-                                  tile it runs). */
+                                  takes 17 (FP32) or 3 (16-bit storage), smaller grids 16. */
 
 /* Propagation kernel selection: AUTO takes the TMA-tiled kernel when it applies (x/y radius
  * 2, theta radius 3, K >= 8, W a multiple of 16 bytes of storage) and the generic one
@@ -311,7 +309,7 @@ loc_status loc_map_difficulty(loc_handle h, const int32_t* probes, int n_probes,
  * finishes a session's last tile sums that session's tile partials into Z in the same fixed
  * order as loc_step's tiled kernel with the same tile configuration, so a session's result
  * does not depend on the other sessions of the batch. */
-#define LOC_BATCH_CONFIGS 3    /* the synchronous tile configurations 1-3 of LOC_TILE_CONFIGS */
+#define LOC_BATCH_CONFIGS 3    /* the tile configurations 1-3 of LOC_TILE_CONFIGS */
 
 /* Group n sessions (distinct handles on one device, one storage type, one stream, each able to
  * use the tiled kernel: default radii, K >= 8, W a multiple of 4 (FP32) or 8 (16-bit)).  The

@@ -1,13 +1,13 @@
 // Batched propagation: many sessions of uneven H x W x K stepped by one persistent launch.
 //
 // The grid is sized to the GPU (resident CTAs per SM x SMs).  Each CTA repeatedly takes the
-// next (session, tile) item from a device work queue and runs the synchronous tiled pass
-// (Algorithm 1's propagation, run_tile) on that session's tile; the CTA that finishes a session's last
+// next (session, tile) item from a device work queue and runs Algorithm 1's propagation on that
+// session's tile (the streaming tiles of stream.cuh, or the synchronous run_tile); the CTA that finishes a session's last
 // tile combines the session's FP64 tile partials into its normaliser Z (Eq. 9) in the same
 // fixed order as a single-session launch, so a session's result does not depend on which
 // other sessions share the launch.
 #include "kernels.h"
-#include "tiled_common.cuh"
+#include "stream.cuh"
 
 namespace loc {
 namespace {
@@ -127,10 +127,76 @@ batch_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restrict__ t
     }
 }
 
-// The candidates: the synchronous tile configurations 1-3 of the single-session kernel.
+// The same queue for the streaming tiles (stream.cuh): the manager warp takes the items, so the
+// next item's planes are in flight while the CTA finishes the previous one.
+template <typename T>
+__global__ void __launch_bounds__(stream::NT, 1)
+batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restrict__ tk, const BatchList* __restrict__ list,
+                    const BatchActive* __restrict__ act, const Shift* __restrict__ shifts, BatchCtl* ctl, int dry) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const uint32_t base = su32(smem_raw);
+    stream::Smem<T>& sm = *reinterpret_cast<stream::Smem<T>*>(smem_raw + (((base + 127u) & ~127u) - base));
+    const int lane = threadIdx.x & 31;
+    const int total = list->total, n_active = list->n_active;
+    stream::run_roles<T, false>(
+        sm,
+        [&](stream::Item& it, stream::Source& src) {
+            int q = 0;
+            if (lane == 0) q = atomicAdd(&ctl->head, 1);
+            q = __shfl_sync(0xffffffffu, q, 0);
+            if (q >= total) return;
+            int lo = 0, hi = n_active - 1;               // last entry with start <= q
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (act[mid].start <= q) lo = mid;
+                else hi = mid - 1;
+            }
+            const int sess = act[lo].s, tile = q - act[lo].start;
+            const int cur = tk[sess].cur;
+            const BatchStatic& S = ss[sess];
+            // a dry run times the steady state (TMA input) whatever the session's restart flag
+            src.reinit = dry ? 0 : S.sd->reinit;
+            src.sh = shifts + S.sh_off;
+            src.tmap = reinterpret_cast<const CUtensorMap*>(S.tmap[cur]);
+            // the tensor map lives in global memory, written by a copy before the launch
+            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(src.tmap) : "memory");
+            it.out = S.B[1 - cur];
+            it.trav = S.trav;
+            it.corr = S.corr;
+            it.K = S.K;
+            it.H = S.H;
+            it.W = S.W;
+            it.ty0 = (tile / S.ntx) * stream::TH;
+            it.tx0 = (tile % S.ntx) * TW;
+            // restart: the input is M / (K n_free); read M and fold 1 / (K n_free) into the scale
+            it.in_scale = (src.reinit ? S.inv_uniform : S.sd->inv_Z) * S.out_mult;
+            it.g0 = S.g0;
+            it.g1 = S.g1;
+            it.g2 = S.g2;
+#pragma unroll
+            for (int d = 0; d < RING; ++d) it.gt[d] = S.gt[d];
+            it.tile = tile;
+            it.ntiles = S.ntiles;
+            it.sd = S.sd;
+            it.partials = S.partials;
+            it.log_out_mult = S.log_out_mult;
+        },
+        [&](const stream::Item& it, int slot) {
+            if (dry) return;
+            stream::retire_tile<false>(sm, it, slot, it.partials, nullptr, nullptr, &it.sd->counter,
+                                       [&](double Z, const ArgBest&) { stream::session_finish(it.sd, Z, it.log_out_mult); });
+        });
+    if (threadIdx.x == 0 && sm.fail) {
+        // flag the launch and the sessions of the tiles in work; their Z is not updated
+        atomicOr(&ctl->status, LOC_DEV_ERR_TIMEOUT);
+        for (int k = 0; k < 2; ++k)
+            if (sm.item[k].K > 0) atomicOr(&sm.item[k].sd->status, LOC_DEV_ERR_TIMEOUT);
+    }
+}
+
+// The candidates: the tile configurations 1-3 of the single-session kernel (3: streaming).
 using BCfg1 = Cfg<32, 4, 3, 16, 3, 2>;
 using BCfg2 = Cfg<16, 2, 2, 8, 3, 3>;
-using BCfg3 = Cfg<16, 4, 4, 16, 3, 4>;
 
 template <typename T, typename C>
 cudaError_t prepare_typed(int* grid) {
@@ -159,11 +225,30 @@ cudaError_t launch_typed(int grid, const BatchStatic* ss, const void* tick, cons
 }
 
 template <typename T>
+cudaError_t prepare_stream(int* grid) {
+    cudaError_t e = stream::prepare<T>(batch_stream_kernel<T>);
+    int dev = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(grid, cudaDevAttrMultiProcessorCount, dev);   // one CTA per SM
+    return e;
+}
+
+template <typename T>
+cudaError_t launch_stream(int grid, const BatchStatic* ss, const void* tick, const BatchLayout& lay, BatchCtl* ctl,
+                          int dry, cudaStream_t st) {
+    const unsigned char* b = static_cast<const unsigned char*>(tick);
+    batch_stream_kernel<T><<<grid, stream::NT, sizeof(stream::Smem<T>) + 128, st>>>(
+        ss, reinterpret_cast<const BatchTick*>(b), reinterpret_cast<const BatchList*>(b + lay.list_off),
+        reinterpret_cast<const BatchActive*>(b + lay.act_off), reinterpret_cast<const Shift*>(b + lay.shifts_off), ctl, dry);
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t prepare_cfg(int cfg, int* grid) {
     switch (cfg) {
         case 1: return prepare_typed<T, BCfg1>(grid);
         case 2: return prepare_typed<T, BCfg2>(grid);
-        case 3: return prepare_typed<T, BCfg3>(grid);
+        case 3: return prepare_stream<T>(grid);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -174,7 +259,7 @@ cudaError_t launch_cfg(int cfg, int grid, const BatchStatic* ss, const void* tic
     switch (cfg) {
         case 1: return launch_typed<T, BCfg1>(grid, ss, tick, lay, ctl, dry, st);
         case 2: return launch_typed<T, BCfg2>(grid, ss, tick, lay, ctl, dry, st);
-        case 3: return launch_typed<T, BCfg3>(grid, ss, tick, lay, ctl, dry, st);
+        case 3: return launch_stream<T>(grid, ss, tick, lay, ctl, dry, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -185,7 +270,7 @@ size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 int batch_num_cfgs() { return 3; }
 
-int batch_tile_rows(int cfg) { return cfg == 1 ? BCfg1::TH : cfg == 2 ? BCfg2::TH : BCfg3::TH; }
+int batch_tile_rows(int cfg) { return cfg == 1 ? BCfg1::TH : cfg == 2 ? BCfg2::TH : stream::TH; }
 
 cudaError_t batch_prepare(int storage, int cfg, int* grid) {
     switch (storage) {

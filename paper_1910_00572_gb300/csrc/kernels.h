@@ -55,11 +55,16 @@ size_t step_tmap_bytes();
 cudaError_t make_step_tmap(void* tmap_out, const void* B, int storage, int H, int W, int K, int cfg);
 // Tensor map of a [K][H][W] belief buffer loaded in boxes of box_w x box_h cells of one plane.
 cudaError_t make_box_tmap(void* tmap_out, const void* B, int storage, int H, int W, int K, int box_w, int box_h);
+// The streaming form (step_stream.cu) of args = tiled::FastArgs, with or without the fused
+// argmax; its tile rows and raw box width (its boxes are tile rows + 5 high).
+cudaError_t launch_step_stream(const void* args, int storage, bool argmax, cudaStream_t st);
+int stream_tile_rows();
+int stream_box_w(int storage);
 cudaError_t launch_step_tiled(const StepArgs& a, const void* tmap, int storage, int cfg, cudaStream_t st);
 
 // ---- Batched propagation (batch.cu): one persistent launch over (session, tile) items of
-// many sessions.  Batch configurations 1 .. batch_num_cfgs() are the synchronous tiled
-// configurations of the same number (same tile rows, same tensor maps).
+// many sessions.  Batch configurations 1 .. batch_num_cfgs() are the tiled configurations of
+// the same number (same tile rows, same tensor maps).
 struct alignas(128) BatchStatic {           // per session, uploaded once
     unsigned char tmap[2][128];             // tensor maps of B[0], B[1] (CUtensorMap)
     void* B[2];

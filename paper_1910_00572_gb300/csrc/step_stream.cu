@@ -1,0 +1,97 @@
+// Single-session launch of the streaming propagation (stream.cuh): the tiles of one grid,
+// dealt to the persistent CTAs in turn.
+#include <type_traits>
+
+#include "stream.cuh"
+
+namespace loc {
+namespace {
+
+using namespace stream;
+
+template <typename T, bool AM>
+__global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid_constant__ FastArgs a, int ntx,
+                                                                    int ntiles) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const uint32_t sbase = su32(smem_raw);
+    stream::Smem<T>& sm = *reinterpret_cast<stream::Smem<T>*>(smem_raw + (((sbase + 127u) & ~127u) - sbase));
+    const int reinit = a.sd->reinit;
+    // restart: the input is M / (K n_free); read M and fold 1 / (K n_free) into the scale
+    const float in_scale = (reinit ? a.inv_uniform : a.sd->inv_Z) * a.out_mult;
+    int tile = blockIdx.x;
+    run_roles<T, AM>(
+        sm,
+        [&](Item& it, Source& src) {
+            if (tile >= ntiles) return;
+            it.out = a.B_out;
+            it.trav = a.trav;
+            it.corr = a.corr;
+            it.K = a.K;
+            it.H = a.H;
+            it.W = a.W;
+            it.ty0 = (tile / ntx) * stream::TH;
+            it.tx0 = (tile % ntx) * TW;
+            it.in_scale = in_scale;
+            it.g0 = a.g0;
+            it.g1 = a.g1;
+            it.g2 = a.g2;
+#pragma unroll
+            for (int d = 0; d < RING; ++d) it.gt[d] = a.gt[d];
+            it.tile = tile;
+            it.ntiles = ntiles;
+            src.tmap = &a.tmap;
+            src.sh = a.sh;
+            src.reinit = reinit;
+            tile += gridDim.x;
+        },
+        [&](const Item& it, int slot) {
+            retire_tile<AM>(sm, it, slot, a.partials, a.am_pv, a.am_pi, &a.sd->counter, [&](double Z, const ArgBest& b) {
+                session_finish(a.sd, Z, a.log_out_mult);
+                if constexpr (AM) {
+                    // no result when the session restarts
+                    const bool live = Z > 0.0 && isfinite(Z);
+                    *a.am_idx = live ? b.i : -1;
+                    if (live) *a.am_val = (float)((double)b.v / Z);
+                }
+            });
+        });
+    if (threadIdx.x == 0 && sm.fail) atomicOr(&a.sd->status, LOC_DEV_ERR_TIMEOUT);
+}
+
+template <typename T, bool AM>
+cudaError_t launch(const FastArgs& a, cudaStream_t st) {
+    static bool attr_set[64] = {};
+    static int sms[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int slot = dev >= 0 && dev < 64 ? dev : 0;
+    const size_t sb = sizeof(stream::Smem<T>) + 128;
+    if (slot != dev || !attr_set[slot]) {
+        cudaError_t e = prepare<T>(step_stream_kernel<T, AM>);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[slot], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        attr_set[slot] = true;
+    }
+    const int ntx = (a.W + TW - 1) / TW, ntiles = ntx * ((a.H + stream::TH - 1) / stream::TH);
+    const int grid = ntiles < sms[slot] ? ntiles : sms[slot];
+    step_stream_kernel<T, AM><<<grid, stream::NT, sb, st>>>(a, ntx, ntiles);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_step_stream(const void* args, int storage, bool argmax, cudaStream_t st) {
+    const FastArgs& a = *static_cast<const FastArgs*>(args);
+    switch (storage) {
+        case LOC_F32: return argmax ? launch<float, true>(a, st) : launch<float, false>(a, st);
+        case LOC_BF16: return argmax ? launch<__nv_bfloat16, true>(a, st) : launch<__nv_bfloat16, false>(a, st);
+        case LOC_F16: return argmax ? launch<__half, true>(a, st) : launch<__half, false>(a, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+int stream_tile_rows() { return stream::TH; }
+
+int stream_box_w(int storage) { return storage == LOC_F32 ? box_w<float>() : box_w<__half>(); }
+
+}  // namespace loc

@@ -15,7 +15,7 @@
 // shared memory (planes p = K .. K+5 read them back), so every input plane is read from HBM
 // once.  CTA partials are combined in FP64 by the last CTA (Z, log-scale).
 //
-// Tile configurations (Cfg1..Cfg16) trade halo overhead against the number of resident CTAs
+// Tile configurations trade halo overhead against the number of resident CTAs
 // and how the passes are spread over warps; the session picks one per grid shape.
 #include <type_traits>
 
@@ -372,11 +372,10 @@ __global__ void __launch_bounds__(C::NT, C::MINB) step_ws_kernel(const __grid_co
                       a.am_val, [sd, log_mult](double Z) { finish_step(sd, Z, log_mult); });
 }
 
-// The tile configurations.  1: 32-row tiles (large grids); 2: 16-row tiles with 2-row
-// P-pass items (256 threads); 3: 16-row tiles with 4-row P-pass items (128 threads).
+// The tile configurations of this file.  1: 32-row tiles; 2: 16-row tiles with 2-row P-pass
+// items (256 threads).  3, 16 and 17 are the streaming kernel (stream.cuh).
 using Cfg1 = Cfg<32, 4, 3, 16, 3, 2>;
 using Cfg2 = Cfg<16, 2, 2, 8, 3, 3>;
-using Cfg3 = Cfg<16, 4, 4, 16, 3, 4>;
 using Cfg4 = Cfg<16, 1, 2, 8, 3, 2>;
 using Cfg5 = Cfg<32, 2, 3, 16, 3, 1>;
 using Cfg6 = WsCfg<16, 4, 16, 3, 2>;   // warp-specialised, 16-row tiles
@@ -389,17 +388,14 @@ using Cfg9 = pairs::PCfg<16, 2, 2, 4, 3, 2>;
 using Cfg10 = pairs::PCfg<32, 4, 2, 8, 2, 2>;
 using Cfg11 = pairs::PCfg<8, 2, 2, 8, 3, 4>;
 using Cfg12 = pairs::PCfg<16, 4, 2, 8, 2, 4>;
-// 13: warp-specialised 14-row tiles (the consumers cover 16 rows, 14 stored); 14-16: split
+// 13: warp-specialised 14-row tiles (the consumers cover 16 rows, 14 stored); 14, 15: split
 // producers (S warps beside X warps): 14: 16-row tiles, 96 + 96 producer threads; 15: 14-row
-// tiles, 64 + 96; 16: 28-row tiles, one CTA of 16 warps per SM (160 + 128 producer threads,
-// 224 consumer threads).
+// tiles, 64 + 96.
 using Cfg13 = WsCfg<14, 3, 16, 3, 2, 128, 128, 4>;
 using Cfg14 = WsCfg<16, 4, 16, 3, 2, 192, 128, 0, true>;
 using Cfg15 = WsCfg<14, 6, 16, 3, 2, 160, 128, 4, true>;
-using Cfg16 = WsCfg<28, 4, 16, 3, 1, 288, 224, 4, true>;
-// 17, 18: configurations 3 and 2 as a software pipeline over the planes (run_tile_pipe: one
-// CTA barrier per plane, S and X double-buffered).
-using Cfg17 = Cfg<16, 4, 4, 16, 3, 3, true>;
+// 18: configuration 2 as a software pipeline over the planes (run_tile_pipe: one CTA barrier
+// per plane, S and X double-buffered).
 using Cfg18 = Cfg<16, 2, 2, 8, 3, 3, true>;
 
 template <typename T, typename C> size_t smem_bytes() {
@@ -443,7 +439,6 @@ cudaError_t launch_cfg(int cfg, const FastArgs& a, int W, int H, cudaStream_t st
     switch (cfg) {
         case 1: return launch_typed<T, Cfg1>(a, dim3((W + TW - 1) / TW, (H + Cfg1::TH - 1) / Cfg1::TH), st);
         case 2: return launch_typed<T, Cfg2>(a, dim3((W + TW - 1) / TW, (H + Cfg2::TH - 1) / Cfg2::TH), st);
-        case 3: return launch_typed<T, Cfg3>(a, dim3((W + TW - 1) / TW, (H + Cfg3::TH - 1) / Cfg3::TH), st);
         case 4: return launch_typed<T, Cfg4>(a, dim3((W + TW - 1) / TW, (H + Cfg4::TH - 1) / Cfg4::TH), st);
         case 5: return launch_typed<T, Cfg5>(a, dim3((W + TW - 1) / TW, (H + Cfg5::TH - 1) / Cfg5::TH), st);
         case 6: return launch_ws<T, Cfg6>(a, dim3((W + TW - 1) / TW, (H + Cfg6::TH - 1) / Cfg6::TH), st);
@@ -456,8 +451,6 @@ cudaError_t launch_cfg(int cfg, const FastArgs& a, int W, int H, cudaStream_t st
         case 13: return launch_ws<T, Cfg13>(a, dim3((W + TW - 1) / TW, (H + Cfg13::TH - 1) / Cfg13::TH), st);
         case 14: return launch_ws<T, Cfg14>(a, dim3((W + TW - 1) / TW, (H + Cfg14::TH - 1) / Cfg14::TH), st);
         case 15: return launch_ws<T, Cfg15>(a, dim3((W + TW - 1) / TW, (H + Cfg15::TH - 1) / Cfg15::TH), st);
-        case 16: return launch_ws<T, Cfg16>(a, dim3((W + TW - 1) / TW, (H + Cfg16::TH - 1) / Cfg16::TH), st);
-        case 17: return launch_typed<T, Cfg17>(a, dim3((W + TW - 1) / TW, (H + Cfg17::TH - 1) / Cfg17::TH), st);
         case 18: return launch_typed<T, Cfg18>(a, dim3((W + TW - 1) / TW, (H + Cfg18::TH - 1) / Cfg18::TH), st);
         default: return cudaErrorInvalidValue;
     }
@@ -467,7 +460,6 @@ int cfg_tile_rows(int cfg) {
     switch (cfg) {
         case 1: return Cfg1::TH;
         case 2: return Cfg2::TH;
-        case 3: return Cfg3::TH;
         case 4: return Cfg4::TH;
         case 5: return Cfg5::TH;
         case 6: return Cfg6::TH;
@@ -480,8 +472,6 @@ int cfg_tile_rows(int cfg) {
         case 13: return Cfg13::TH;
         case 14: return Cfg14::TH;
         case 15: return Cfg15::TH;
-        case 16: return Cfg16::TH;
-        case 17: return Cfg17::TH;
         default: return Cfg18::TH;
     }
 }
@@ -512,6 +502,9 @@ bool step_tiled_eligible(int H, int W, int K, int r_xy, int r_th, int storage) {
 
 int step_tiled_num_cfgs() { return 18; }
 
+// Configurations that run the streaming kernel (stream.cuh)
+static bool is_stream_cfg(int cfg) { return cfg == 3 || cfg == 16 || cfg == 17; }
+
 bool step_tiled_fuses_argmax(int cfg) { return cfg == 6 || cfg == 7 || (cfg >= 13 && cfg <= 16); }
 
 int step_tiled_default_cfg(int H, int W, int K, int storage) {
@@ -520,30 +513,20 @@ int step_tiled_default_cfg(int H, int W, int K, int storage) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         nsm = 152;
-    // measured on GB300 (office plans): with many tiles per SM the 128-thread synchronous
-    // configuration (3) is fastest for 16-bit storage, and its software-pipelined form (17, three
-    // CTAs per SM) for FP32 (2048 x 2048 x 72: 0.79 against 0.83 ms; BF16 0.81 against 0.73)
+    // The streaming kernel on every grid (64 x 64 x 16 to 2048 x 2048 x 72: 0.64 to 0.79 of the
+    // time of the tile configurations it took the place of).  The argmax is combined in the step
+    // (16) where a pose is likely to be read after every step and the step is short: it costs
+    // 4 us at 512 x 512 x 64 (43 against 39), the pass it saves 17; on grids of at least 8
+    // sixteen-row tiles per SM it is left to the pass (17 for FP32, 3 for 16-bit storage).
     const long long cols = (W + TW - 1) / TW;
     if (cols * ((H + 15) / 16) >= 8LL * nsm) return storage == LOC_F32 ? 17 : 3;
-    // with few tiles the warp-specialised pipelines, whose time follows the S/X rows (tile rows
-    // + 4) that the busiest SM computes: 16-row tiles two per SM (6), 14-row tiles two per SM
-    // with split producers (15), 28-row tiles one per SM (16); ties keep the earlier one
-    const int cand[3][2] = {{6, Cfg6::TH}, {15, Cfg15::TH}, {16, Cfg16::TH}};
-    int best = 6;
-    long long best_cost = -1;
-    for (const auto& c : cand) {
-        const long long tiles = cols * ((H + c[1] - 1) / c[1]);
-        const long long cost = (tiles + nsm - 1) / nsm * (c[1] + 2 * R);
-        if (best_cost < 0 || cost < best_cost) {
-            best = c[0];
-            best_cost = cost;
-        }
-    }
-    return best;
+    return 16;
 }
 
 cudaError_t make_step_tmap(void* tmap_out, const void* B, int storage, int H, int W, int K, int cfg) {
     if (cfg < 1 || cfg > step_tiled_num_cfgs()) return cudaErrorInvalidValue;
+    if (is_stream_cfg(cfg))
+        return make_box_tmap(tmap_out, B, storage, H, W, K, stream_box_w(storage), stream_tile_rows() + 2 * R + 1);
     const bool paired = cfg >= 8 && cfg <= 12;    // the paired-column passes use a wider box
     const int bw = !paired ? BW : (storage == LOC_F32 ? pairs::pbw<float>() : pairs::pbw<__half>());
     return make_box_tmap(tmap_out, B, storage, H, W, K, bw, cfg_tile_rows(cfg) + 2 * R + 1);
@@ -591,6 +574,7 @@ cudaError_t launch_step_tiled(const StepArgs& g, const void* tmap, int storage, 
     a.g2 = g.gx[R + 2];
     for (int d = 0; d < RING; ++d) a.gt[d] = g.gt[d];
     for (int k = 0; k < g.K; ++k) a.sh[k] = g.sh[k];
+    if (is_stream_cfg(cfg)) return launch_step_stream(&a, storage, step_tiled_fuses_argmax(cfg), st);
     cudaError_t e;
     switch (storage) {
         case LOC_F32: e = launch_cfg<float>(cfg, a, g.W, g.H, st); break;
