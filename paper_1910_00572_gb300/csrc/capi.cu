@@ -174,6 +174,8 @@ LOC_API loc_status loc_session_bytes(const loc_params* p, size_t* bytes) {
     size_t cap = 2 * (size_t)p->n_samples + 4 * (H + W) + 1024;
     if (cap > hw) cap = hw;
     const size_t nrb = (H + 31) / 32;
+    // (the selections take an eighth of the hw bytes counted for them: room for the tables that a
+    // scan of more beams grows)
     b += r(hw * 4) + r(hw) + 2 * r(H * 4) + r((nrb + 1) * W * 4) + r((nrb + 2) * 4) + r(cap * 4) +
          r(cap * K * 4) + r(64) + r(reweight_scalars_bytes()) + r(K * 1080 * 8) + r(1080 * 4) + r(K * 1080 * 4) +
          r(H * ((W + 31) / 32) * 4);
@@ -420,16 +422,15 @@ loc_status lidar_setup(loc_session* h) {
     const int nrb = (H + 31) / 32;
     h->m = (float*)dev_alloc(h, sizeof(float) * hw);
     h->travbits = (uint32_t*)dev_alloc(h, sizeof(uint32_t) * (size_t)H * ((W + 31) / 32));
-    h->sel = (uint8_t*)dev_alloc(h, hw);
+    h->sel = (uint32_t*)dev_alloc(h, sizeof(uint32_t) * (size_t)H * ((W + 31) / 32));
     h->rowcnt = (int*)dev_alloc(h, sizeof(int) * H);
     h->rowoff = (int*)dev_alloc(h, sizeof(int) * H);
     h->bnd = (float*)dev_alloc(h, sizeof(float) * (size_t)(nrb + 1) * W);
-    h->prog = (int*)dev_alloc(h, sizeof(int) * (size_t)(nrb + 2));
     h->samples = (int32_t*)dev_alloc(h, sizeof(int32_t) * (size_t)cap);
     h->logL = (float*)dev_alloc(h, sizeof(float) * (size_t)cap * K);
     h->dscal = (int*)dev_alloc(h, 64);
     h->rs = dev_alloc(h, reweight_scalars_bytes());
-    if (!h->m || !h->sel || !h->rowcnt || !h->rowoff || !h->bnd || !h->prog || !h->samples || !h->logL ||
+    if (!h->m || !h->sel || !h->rowcnt || !h->rowoff || !h->bnd || !h->samples || !h->logL ||
         !h->dscal || !h->rs || !h->travbits)
         return fail(h, LOC_ERR_OOM, "LIDAR scratch allocation failed");
     cudaError_t e = cudaMemsetAsync(h->dscal, 0, 64, h->stream);
@@ -643,7 +644,7 @@ LOC_API loc_status loc_lidar_update(loc_handle h, const float* ranges, int n_bea
                                       reinterpret_cast<float*>(h->dscal + 2), h->stream);
     if (e == cudaSuccess)
         e = launch_dither(h->m, reinterpret_cast<float*>(h->dscal + 2), h->p.H, h->p.W, h->sel, h->rowcnt,
-                          h->rowoff, h->dscal, h->bnd, h->prog, &h->sd->status, h->cap, h->samples, h->stream);
+                          h->rowoff, h->dscal, h->bnd, &h->sd->status, h->cap, h->samples, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sample selection launch");
     return score_and_reweight(h, nu, nd, r_max, sigma_r);
 }
@@ -721,11 +722,16 @@ LOC_API loc_status loc_dither(loc_handle h, const float* m, float fs, uint8_t* s
         e = cudaMemcpyAsync(h->dscal + 2, &fs, sizeof(float), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
         e = launch_dither(h->m, reinterpret_cast<float*>(h->dscal + 2), h->p.H, h->p.W, h->sel, h->rowcnt, h->rowoff,
-                          h->dscal + 3, h->bnd, h->prog, &h->sd->status, 0, nullptr, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sel, h->sel, h->hw, cudaMemcpyDeviceToHost, h->stream);
+                          h->dscal + 3, h->bnd, &h->sd->status, 0, nullptr, h->stream);
+    const int H = h->p.H, W = h->p.W, nch = (W + 31) / 32;
+    std::vector<uint32_t> bits((size_t)H * nch);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(bits.data(), h->sel, sizeof(uint32_t) * bits.size(), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(count, h->dscal + 3, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_dither");
+    for (int j = 0; j < H; ++j)
+        for (int i = 0; i < W; ++i) sel[(size_t)j * W + i] = (bits[(size_t)j * nch + (i >> 5)] >> (i & 31)) & 1u;
     return sync_and_check(h);
 }
 

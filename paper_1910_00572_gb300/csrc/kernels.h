@@ -156,12 +156,11 @@ cudaError_t launch_set_belief(const float* src, void* B, int storage, size_t n,
 cudaError_t launch_belief_map(const void* B, int storage, const uint8_t* trav, SessionDev* sd, float inv_uniform,
                               int H, int W, int K, float* m, double* partials, unsigned int nparts,
                               unsigned int* counter, int n_samples, float* fs_out, cudaStream_t st);
-// Floyd-Steinberg selection of m * fs -> sel, per-row counts/offsets, total -> *count and (if
-// samples) the raster-ordered list of at most cap selected linear indices.  bnd holds
-// ((H+31)/32 + 1) * W floats, prog (H+31)/32 + 2 ints.
-cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint8_t* sel, int* rowcnt, int* rowoff,
-                          int* count, float* bnd, int* prog, int* status, int cap, int32_t* samples,
-                          cudaStream_t st);
+// Floyd-Steinberg selection of m * fs -> selbits (row j: ceil(W / 32) words, bit b of word w =
+// cell (j, 32 w + b) is selected), per-row counts/offsets, total -> *count and (if samples) the
+// raster-ordered list of at most cap selected linear indices.  bnd holds ceil(H / 32) * W floats.
+cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_t* selbits, int* rowcnt, int* rowoff,
+                          int* count, float* bnd, int* status, int cap, int32_t* samples, cudaStream_t st);
 cudaError_t launch_ray_ranges(const uint8_t* trav, int H, int W, const int32_t* cells, int n_cells, const float* dirs,
                               int n_dirs, float rmax_cells, float cell_m, float* out, cudaStream_t st);
 size_t reweight_scalars_bytes();

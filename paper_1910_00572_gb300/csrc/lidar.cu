@@ -102,85 +102,77 @@ __global__ void __launch_bounds__(NT) belief_map_vec_kernel(const T* __restrict_
 
 // ------------------------------------------------------------------ Floyd-Steinberg
 
-// One CTA of kFsWarps warps.  Warp w takes the 32-row blocks rb = w, w + kFsWarps, ...; lane l
-// owns row 32 rb + l and handles column i = t - 2l at step t, so the three errors it needs from
-// the row above (columns i-1, i, i+1) were produced by lane l-1 at steps t-3, t-2, t-1 and
-// arrive by warp shuffle.  Lane 0 takes the row above from the previous block's last row,
-// which that block's lane 31 writes into bnd[rb][*] and publishes in prog[rb] (columns
-// written); every wait on prog is bounded.
+// Warp w of a cluster of kFsWarps-warp CTAs takes the 32-row blocks w, w + (all warps), ...; lane l
+// owns row 32 rb + l and handles column i = t - 3 l at step t.  The three errors it needs from the
+// row above (columns i - 1, i, i + 1) were produced by lane l - 1 at steps t - 4, t - 3 and t - 2
+// and arrive by warp shuffle one step before they are used, so only the lane's own error chain
+// (multiply, two adds, compare) is left between two steps.
 //
-// Each warp keeps a ring of three 32-column chunks per row in shared memory (column i at
-// position i mod 96).  A lane reads min(1, m fs) of its cell there and writes its selection
-// back in its place.  Steps run in windows of 32: at step 32 T the last lane has finished chunk
-// T - 3 (at step 32 T - 3), so the warp copies that chunk's selections to sel (each lane its own
-// row) and stores chunk T of the map (loaded into registers, coalesced, one window earlier) in
-// its place.  Terms of the error sum whose source lies outside the grid are zero (their errors
-// were never produced), so the sum always takes the same four terms in the same order; only
-// the right neighbour above is masked at the last column.
+// What bounds it: the chain.  A row can take column i only when the row above has taken i + 1, so
+// the whole map is a wavefront of W + 94 + (blocks - 1) x (94 + hand-off) steps.  One CTA of 16
+// warps (four rows of blocks one after the other, 16 warps on four schedulers, a fence per
+// hand-off) took 1.73 ms at 2048 x 2048; a warp per block on a scheduler of its own, with
+// hand-offs that need no fence, takes FSUS.  The cluster keeps the warps that wait on one another
+// resident together.
+//
+// Hand-off: a block's last lane writes its errors to bnd[rb + 1][*] as it goes.  The whole buffer
+// starts as kFsEmpty (a NaN that no arithmetic produces), so a value that is not kFsEmpty is
+// there: the next block polls the 32 values of its window themselves, with a limit.
+//
+// Each warp keeps a ring of four 32-column chunks per row in shared memory (column i at position
+// i mod 128), the first chunk repeated behind the fourth so that a window of 32 steps reads at
+// constant offsets; a pitch of 162 makes the lanes' 3-column skew hit distinct banks.  At step
+// 32 T the last lane has finished chunk T - 4, so chunk T of the map (loaded into registers,
+// coalesced, one window earlier) takes its place.  Selections are bits: a lane collects a window's
+// 32 and writes them as one aligned word of its row.  Terms of the error sum whose source lies
+// outside the grid are zero (their errors were never produced), so the sum always takes the same
+// four terms in the same order; only the right neighbour above is masked at the last column.
 constexpr size_t kScoreWindowBytes = 96 * 1024;   // shared memory for the score kernel's map window
 constexpr int kScoreNT = 384;                      // score kernel threads: 360 beam directions in one round
-constexpr int kFsWarps = 16;
-constexpr int kFsPitch = 97;              // 3 x 32 columns + 1: lane accesses hit distinct banks
+constexpr int kFsWarps = 4;               // one per scheduler
+constexpr int kFsMaxCtas = 16;            // largest cluster: 64 blocks of 32 rows side by side
+constexpr int kFsSkew = 3;
+constexpr int kFsLead = 32 * kFsSkew;     // steps of skew over a block, rounded up: 93 -> 96
+constexpr int kFsPitch = 162;
+constexpr uint32_t kFsEmpty = 0xFFFFFFFFu;
 
 __global__ void __launch_bounds__(kFsWarps * 32) fs_kernel(const float* __restrict__ m, const float* fs_ptr, int H,
-                                                           int W, uint8_t* __restrict__ sel, int* __restrict__ rowcnt,
-                                                           float* bnd, int* prog, int* status) {
+                                                           int W, uint32_t* __restrict__ selbits,
+                                                           int* __restrict__ rowcnt, float* bnd, int* status) {
     extern __shared__ float fs_ring_all[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* ring = fs_ring_all + (size_t)warp * 32 * kFsPitch;
-    float* own = ring + lane * kFsPitch;                       // this lane's row
+    const float* own = ring + lane * kFsPitch;                 // this lane's row
     const float fs = *fs_ptr;
     const unsigned long long wait_ns = g_fs_wait_ns;
     const int stall = g_fs_stall;
     const int nrb = (H + 31) / 32, nch = (W + 31) / 32;
-    const int vec = (W & 3) == 0 ? 4 : 1;
     const float w7 = 0.4375f, w3 = 0.1875f, w5 = 0.3125f, w1 = 0.0625f;
-    for (int rb = warp; rb < nrb; rb += kFsWarps) {
+    for (int rb = blockIdx.x * kFsWarps + warp; rb < nrb; rb += gridDim.x * kFsWarps) {
         const int j0 = 32 * rb, j = j0 + lane;
         const bool row_ok = j < H;
-        float pre[32];                                         // column 32 c + lane of rows j0 ..
         const bool interior = j0 + 31 < H;                     // every row of the block in the grid
+        float pre[32];                                         // column 32 c + lane of rows j0 ..
         auto load_chunk = [&](int c) {
             const int col = 32 * c + lane;
             if (interior && col < W) {
                 const float* src = m + (size_t)j0 * W + col;
 #pragma unroll
-                for (int r = 0; r < 32; ++r) pre[r] = src[(size_t)r * W];
+                for (int r = 0; r < 32; ++r) pre[r] = __ldg(src + (size_t)r * W);
             } else {
 #pragma unroll
                 for (int r = 0; r < 32; ++r)
-                    pre[r] = (j0 + r < H && col < W) ? m[(size_t)(j0 + r) * W + col] : 0.0f;
+                    pre[r] = (j0 + r < H && col < W) ? __ldg(m + (size_t)(j0 + r) * W + col) : 0.0f;
             }
         };
         auto store_chunk = [&](int c) {
-            float* dst = ring + (c % 3) * 32 + lane;
+            float* dst = ring + (c & 3) * 32 + lane;
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
                 float v = __fmul_rn(pre[r], fs);
                 if (v > 1.0f) v = 1.0f;
                 dst[r * kFsPitch] = v;
-            }
-        };
-        int cnt = 0;
-        auto copy_out = [&](int c) {                           // this lane's selections of chunk c
-            const float* src = own + (c % 3) * 32;
-            const int c0 = 32 * c, n = min(32, W - c0);
-            uint8_t* out = sel + (size_t)j * W + c0;
-            if (!row_ok) return;
-            if (vec == 4) {
-                for (int k = 0; k < n; k += 4) {
-                    const uint32_t b = (uint32_t)__float_as_uint(src[k]) | ((uint32_t)__float_as_uint(src[k + 1]) << 8) |
-                                       ((uint32_t)__float_as_uint(src[k + 2]) << 16) |
-                                       ((uint32_t)__float_as_uint(src[k + 3]) << 24);
-                    *reinterpret_cast<uint32_t*>(out + k) = b;
-                    cnt += __popc(b);
-                }
-            } else {
-                for (int k = 0; k < n; ++k) {
-                    const uint32_t b = __float_as_uint(src[k]);
-                    out[k] = (uint8_t)b;
-                    cnt += (int)b;
-                }
+                if ((c & 3) == 0) dst[r * kFsPitch + 128] = v;
             }
         };
         __syncwarp();                                          // the previous block's reads are done
@@ -189,118 +181,112 @@ __global__ void __launch_bounds__(kFsWarps * 32) fs_kernel(const float* __restri
         if (nch > 1) load_chunk(1);
         __syncwarp();
         float up_old = 0.0f, up_mid = 0.0f, up_new = 0.0f;   // row above: columns i-1, i, i+1
-        float e_prev = 0.0f, last = 0.0f;                      // own error at i-1; newest error
+        float pend = 0.0f;                                     // ... and the next one, for the next step
+        float last = 0.0f;                                     // own error at the column before
         float chunk = 0.0f;                                    // lane L: bnd[rb][t0 + 1 + L]
-        bool failed = false;
+        uint32_t before = 0;                                   // the previous window's selections
+        int cnt = 0;
+        const int r_off = (kFsLead - kFsSkew * lane) & 31;     // (t0 - 3 lane) mod 32, t0 a multiple of 32
         const bool publish = lane == 31 && rb + 1 < nrb;       // the next block reads this row
-        float* bnd_next = publish ? bnd + (size_t)(rb + 1) * W : bnd;
-        const int steps = W + 62;
-        const int nwin = (steps + 31) / 32;
-        int ri = (96 - 2 * lane) % 96;                         // (t - 2 lane) mod 96
+        float* bnd_next = bnd + (size_t)(rb + 1 < nrb ? rb + 1 : rb) * W;
+        const volatile uint32_t* above = reinterpret_cast<const volatile uint32_t*>(bnd) + (size_t)rb * W;
+        const int nwin = (W + kFsSkew * 31 + 31) / 32;
         for (int T = 0; T < nwin; ++T) {
             const int t0 = 32 * T;
             if (rb > 0) {
-                // the row above for columns t0+1 .. t0+32 must be published before lane 0 uses it
-                const int need = min(W, t0 + 33);
-                int ok = 1;
-                if (lane == 0) {
-                    const unsigned long long g0 = gtime();
-                    unsigned int it = 0;
-                    while (stall || ((volatile int*)prog)[rb] < need) {
-                        if (++it > (1u << 26) || gtime() - g0 > wait_ns) {
-                            ok = 0;
-                            break;
-                        }
+                // the row above, columns t0 + 1 .. t0 + 32 (and column 0 before the first step:
+                // lane 0 starts there at once; other lanes shift theirs in while they wait)
+                const int c = t0 + 1 + lane;
+                uint32_t v = 0u, v0 = 0u;
+                const unsigned long long g0 = gtime();
+                unsigned int it = 0;
+                bool ok;
+                for (;;) {
+                    if (c < W) v = above[c];
+                    if (T == 0) v0 = above[0];
+                    ok = !stall && v != kFsEmpty && v0 != kFsEmpty;
+                    if (__all_sync(0xffffffffu, ok)) break;
+                    if (__any_sync(0xffffffffu, ++it > (1u << 22) || gtime() - g0 > wait_ns)) {
+                        if (lane == 0) atomicOr(status, LOC_DEV_ERR_TIMEOUT);
+                        return;                                // the blocks below run into their limits too
                     }
                 }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) {
-                    failed = true;
-                    if (lane == 0) atomicOr(status, LOC_DEV_ERR_TIMEOUT);
-                    break;
-                }
-                __threadfence_block();
-                const int c = t0 + 1 + lane;
-                chunk = c < W ? ((volatile float*)bnd)[(size_t)rb * W + c] : 0.0f;
-                // lane 0 starts at column 0 at once: the row above at column 0 must already be
-                // in its register chain (other lanes shift theirs in while they wait to start)
-                if (T == 0 && lane == 0) up_new = ((volatile float*)bnd)[(size_t)rb * W];
+                chunk = __uint_as_float(v);
+                if (T == 0 && lane == 0) up_new = __uint_as_float(v0);
             }
-            if (T >= 3 && T - 3 < nch) copy_out(T - 3);
             if (T > 0 && T < nch) {
-                __syncwarp();                                  // chunk T - 3 is read and copied
+                __syncwarp();                                  // chunk T - 4 is read
                 store_chunk(T);
                 __syncwarp();
                 if (T + 1 < nch) load_chunk(T + 1);
             }
-            if (interior && t0 >= 62 && t0 + 31 <= W - 2) {
-                // Every lane's column lies in [0, W - 2] for the whole window and every row of the
-                // block is in the grid: no column or row guards, the right neighbour above always
-                // exists, and lane 31 publishes its progress once, after the window.  The same
-                // operations in the same order as the general steps below (0 + x == x exactly,
-                // and chunk is 0 when there is no row above).
+            const float* ow = own + ((t0 - kFsSkew * lane) & 127);
+            uint32_t bits = 0;
+            if (interior && t0 >= kFsSkew * 31 && t0 + 31 <= W - 2) {
+                // every lane's column lies in [0, W - 2] for the whole window and every row of the
+                // block is in the grid: no guards.  The same operations in the same order as the
+                // general steps below (0 + x == x exactly, and chunk is 0 with no row above).
 #pragma unroll
                 for (int s = 0; s < 32; ++s) {
                     const float from_above = __shfl_sync(0xffffffffu, chunk, s);
-                    const float from_left = __shfl_up_sync(0xffffffffu, last, 1);
                     up_old = up_mid;
                     up_mid = up_new;
-                    up_new = lane == 0 ? from_above : from_left;
-                    const float v = own[ri];
+                    up_new = lane == 0 ? from_above : pend;
+                    pend = __shfl_up_sync(0xffffffffu, last, 1);
+                    const float v = ow[s];
                     float E = __fmul_rn(up_old, w1);
                     E = __fadd_rn(E, __fmul_rn(up_mid, w5));
                     E = __fadd_rn(E, __fmul_rn(up_new, w3));
-                    E = __fadd_rn(E, __fmul_rn(e_prev, w7));
-                    const float val = __fadd_rn(v, E);
-                    const bool on = val >= 0.5f;
-                    const float err = on ? __fsub_rn(val, 1.0f) : val;
-                    own[ri] = __uint_as_float(on ? 1u : 0u);
-                    e_prev = err;
-                    last = err;
-                    if (publish) bnd_next[t0 + s - 62] = err;
-                    ri = ri == 95 ? 0 : ri + 1;
+                    E = __fadd_rn(E, __fmul_rn(last, w7));
+                    float val = __fadd_rn(v, E);
+                    if (val >= 0.5f) {
+                        val = __fsub_rn(val, 1.0f);
+                        bits |= 1u << s;
+                    }
+                    last = val;
+                    if (publish) *reinterpret_cast<volatile float*>(bnd_next + t0 + s - kFsSkew * 31) = val;
                 }
-                if (publish) {
-                    __threadfence_block();
-                    ((volatile int*)prog)[rb + 1] = t0 - 30;      // columns 0 .. t0 - 31 written
-                }
-                continue;
-            }
-#pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                const float from_above = __shfl_sync(0xffffffffu, chunk, s);
-                const float from_left = __shfl_up_sync(0xffffffffu, last, 1);
-                const float incoming = lane == 0 ? (rb > 0 ? from_above : 0.0f) : from_left;
-                up_old = up_mid;
-                up_mid = up_new;
-                up_new = incoming;
-                const int i = t0 + s - 2 * lane;
-                const float v = own[ri];
-                if ((unsigned)i < (unsigned)W && row_ok) {
-                    float E = __fadd_rn(0.0f, __fmul_rn(up_old, w1));
-                    E = __fadd_rn(E, __fmul_rn(up_mid, w5));
-                    E = __fadd_rn(E, __fmul_rn(i + 1 < W ? up_new : 0.0f, w3));
-                    E = __fadd_rn(E, __fmul_rn(e_prev, w7));
-                    const float val = __fadd_rn(v, E);
-                    const bool on = val >= 0.5f;
-                    const float err = on ? __fsub_rn(val, 1.0f) : val;
-                    own[ri] = __uint_as_float(on ? 1u : 0u);
-                    e_prev = err;
-                    last = err;
-                    if (lane == 31 && rb + 1 < nrb) {
-                        bnd[(size_t)(rb + 1) * W + i] = err;
-                        if (((i + 1) & 31) == 0 || i == W - 1) {
-                            __threadfence_block();
-                            ((volatile int*)prog)[rb + 1] = i + 1;
+            } else {
+#pragma unroll 4
+                for (int s = 0; s < 32; ++s) {
+                    const float from_above = __shfl_sync(0xffffffffu, chunk, s);
+                    up_old = up_mid;
+                    up_mid = up_new;
+                    up_new = lane == 0 ? (rb > 0 ? from_above : 0.0f) : pend;
+                    pend = __shfl_up_sync(0xffffffffu, last, 1);
+                    const int i = t0 + s - kFsSkew * lane;
+                    const float v = ow[s];
+                    if ((unsigned)i < (unsigned)W && row_ok) {
+                        float E = __fadd_rn(0.0f, __fmul_rn(up_old, w1));
+                        E = __fadd_rn(E, __fmul_rn(up_mid, w5));
+                        E = __fadd_rn(E, __fmul_rn(i + 1 < W ? up_new : 0.0f, w3));
+                        E = __fadd_rn(E, __fmul_rn(last, w7));
+                        float val = __fadd_rn(v, E);
+                        if (val >= 0.5f) {
+                            val = __fsub_rn(val, 1.0f);
+                            bits |= 1u << s;
                         }
+                        last = val;
+                        if (publish) *reinterpret_cast<volatile float*>(bnd_next + i) = val;
                     }
                 }
-                ri = ri == 95 ? 0 : ri + 1;
+            }
+            // the aligned word that this window completes: columns t0 - 3 lane - r_off ..
+            const int c = (t0 - kFsSkew * lane - r_off) >> 5;
+            const uint32_t word = __funnelshift_l(before, bits, r_off);
+            before = bits;
+            if (row_ok && c >= 0 && c < nch) {
+                selbits[(size_t)j * nch + c] = word;
+                cnt += __popc(word);
             }
         }
-        if (failed) return;
-        __syncwarp();
-        for (int c = max(0, nwin - 3); c < nch; ++c) copy_out(c);   // chunks not copied in the loop
+        // the word that a lane's last window began, where it lies in the grid
+        const int c = (32 * nwin - kFsSkew * lane - r_off) >> 5;
+        if (row_ok && r_off > 0 && c >= 0 && c < nch) {
+            const uint32_t word = before >> (32 - r_off);
+            selbits[(size_t)j * nch + c] = word;
+            cnt += __popc(word);
+        }
         if (row_ok) rowcnt[j] = cnt;
     }
 }
@@ -333,21 +319,28 @@ __global__ void __launch_bounds__(1024) row_scan_kernel(const int* __restrict__ 
     if (threadIdx.x == 1023) *count = part[1023];
 }
 
-// Linear indices of the selected cells in raster order (one warp per row), at most cap.
-__global__ void __launch_bounds__(NT) compact_kernel(const uint8_t* __restrict__ sel, const int* __restrict__ rowoff,
+// Linear indices of the selected cells in raster order (one warp per row, a word of 32 selections
+// a lane), at most cap.
+__global__ void __launch_bounds__(NT) compact_kernel(const uint32_t* __restrict__ selbits, const int* __restrict__ rowoff,
                                                      int H, int W, int cap, int32_t* __restrict__ out,
                                                      const int* status) {
     if (*(volatile const int*)status & LOC_DEV_ERR_TIMEOUT) return;   // no row offsets were made
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, nch = (W + 31) / 32;
     for (int j = (blockIdx.x * NT + threadIdx.x) >> 5; j < H; j += (gridDim.x * NT) >> 5) {
         int base = rowoff[j];
-        for (int i0 = 0; i0 < W; i0 += 32) {
-            const int i = i0 + lane;
-            const bool on = i < W && sel[(size_t)j * W + i];
-            const unsigned int ball = __ballot_sync(0xffffffffu, on);
-            const int pos = base + __popc(ball & ((1u << lane) - 1u));
-            if (on && pos >= 0 && pos < cap) out[pos] = j * W + i;
-            base += __popc(ball);
+        for (int c0 = 0; c0 < nch; c0 += 32) {
+            uint32_t w = c0 + lane < nch ? selbits[(size_t)j * nch + c0 + lane] : 0u;
+            const int n = __popc(w);
+            int pos = n;                                       // inclusive prefix over the lanes
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, pos, o);
+                if (lane >= o) pos += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, pos, 31);
+            pos += base - n;
+            for (; w; w &= w - 1, ++pos)
+                if (pos >= 0 && pos < cap) out[pos] = j * W + 32 * (c0 + lane) + __ffs(w) - 1;
+            base += total;
         }
     }
 }
@@ -613,11 +606,10 @@ cudaError_t launch_belief_map(const void* B, int storage, const uint8_t* trav, S
     return cudaGetLastError();
 }
 
-cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint8_t* sel, int* rowcnt, int* rowoff,
-                          int* count, float* bnd, int* prog, int* status, int cap, int32_t* samples,
-                          cudaStream_t st) {
+cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_t* selbits, int* rowcnt, int* rowoff,
+                          int* count, float* bnd, int* status, int cap, int32_t* samples, cudaStream_t st) {
     const int nrb = (H + 31) / 32;
-    cudaError_t e = cudaMemsetAsync(prog, 0, sizeof(int) * (size_t)(nrb + 1), st);
+    cudaError_t e = cudaMemsetAsync(bnd, 0xFF, sizeof(float) * (size_t)nrb * W, st);   // kFsEmpty
     if (e != cudaSuccess) return e;
     const size_t smem = sizeof(float) * kFsWarps * 32 * kFsPitch;
     static bool attr_set[64] = {};
@@ -625,13 +617,28 @@ cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint8_t
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
         e = cudaFuncSetAttribute(fs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fs_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    fs_kernel<<<1, kFsWarps * 32, smem, st>>>(m, fs, H, W, sel, rowcnt, bnd, prog, status);
+    int ctas = 1;                                              // a power of two, one warp per block
+    while (ctas < kFsMaxCtas && ctas * kFsWarps < nrb) ctas *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kFsWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, fs_kernel, m, fs, H, W, selbits, rowcnt, bnd, status);
+    if (e != cudaSuccess) return e;
     row_scan_kernel<<<1, 1024, 0, st>>>(rowcnt, H, rowoff, count, status);
     if (samples)
-        compact_kernel<<<grid_for((size_t)H * 32, 1024), NT, 0, st>>>(sel, rowoff, H, W, cap, samples, status);
+        compact_kernel<<<grid_for((size_t)H * 32, 1024), NT, 0, st>>>(selbits, rowoff, H, W, cap, samples, status);
     return cudaGetLastError();
 }
 

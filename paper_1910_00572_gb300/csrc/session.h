@@ -44,11 +44,10 @@ struct loc_session {
     int cap = 0;                   // capacity of the sample list
     float* m = nullptr;            // belief map [H][W]
     uint32_t* travbits = nullptr;  // the map as bits [H][ceil(W / 32)] (the ray casts' window)
-    uint8_t* sel = nullptr;        // selection mask [H][W]
+    uint32_t* sel = nullptr;       // selections as bits [H][ceil(W / 32)]
     int* rowcnt = nullptr;         // per-row selections [H]
     int* rowoff = nullptr;         // exclusive prefix [H]
     float* bnd = nullptr;          // row-block boundary rows for the dithering wavefront
-    int* prog = nullptr;           // their progress counters
     int32_t* samples = nullptr;    // sampled cells [cap]
     float* logL = nullptr;         // log-likelihood [cap][K]
     int* dscal = nullptr;          // device scalars: count, maxL (as uint), fs (as float)
