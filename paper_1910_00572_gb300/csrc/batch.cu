@@ -138,7 +138,7 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
     stream::Smem<T>& sm = *reinterpret_cast<stream::Smem<T>*>(smem_raw + (((base + 127u) & ~127u) - base));
     const int lane = threadIdx.x & 31;
     const int total = list->total, n_active = list->n_active;
-    stream::run_roles<T, false>(
+    stream::run_roles<T, false, false>(
         sm,
         [&](stream::Item& it, stream::Source& src) {
             int q = 0;

@@ -270,6 +270,7 @@ LOC_API loc_status loc_create(const uint8_t* occ, const loc_params* p, loc_handl
         return fail(nullptr, LOC_ERR_OOM, "pinned host allocation failed");
     }
     s->tiled = tiled_ok && p->kernel != LOC_KERNEL_GENERIC;
+    s->ragged = !s->tiled && !aniso && p->kernel == LOC_KERNEL_AUTO && step_ragged_eligible(p->K, rxy, rth);
     if (aniso && aniso_tma_eligible(p->W, p->storage)) {
         s->aniso_tma = true;
         for (int b = 0; b < 2; ++b) {
@@ -400,8 +401,9 @@ LOC_API loc_status loc_step(loc_handle h, double u, double v, double w) {
         a.sigma_c = (float)h->p.sigma_cross_cells;
         e = launch_step_aniso(a, h->aniso_tma ? h->tmap[h->cur] : nullptr, h->p.storage, h->stream);
     } else {
-        e = h->tiled ? launch_step_tiled(a, h->tmap[h->cur], h->p.storage, h->tile_cfg, h->stream)
-                     : launch_step(a, h->p.storage, h->stream);
+        e = h->tiled    ? launch_step_tiled(a, h->tmap[h->cur], h->p.storage, h->tile_cfg, h->stream)
+            : h->ragged ? launch_step_ragged(a, h->p.storage, h->stream)
+                        : launch_step(a, h->p.storage, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
     step_done(h);

@@ -58,6 +58,10 @@ cudaError_t make_box_tmap(void* tmap_out, const void* B, int storage, int H, int
 // The streaming form (step_stream.cu) of args = tiled::FastArgs, with or without the fused
 // argmax; its tile rows and raw box width (its boxes are tile rows + 5 high).
 cudaError_t launch_step_stream(const void* args, int storage, bool argmax, cudaStream_t st);
+// The same for any row width (no tensor map), x/y radius 2, theta radius 3 and K >= 8, without the
+// fused argmax.
+bool step_ragged_eligible(int K, int r_xy, int r_th);
+cudaError_t launch_step_ragged(const StepArgs& a, int storage, cudaStream_t st);
 int stream_tile_rows();
 int stream_box_w(int storage);
 cudaError_t launch_step_tiled(const StepArgs& a, const void* tmap, int storage, int cfg, cudaStream_t st);

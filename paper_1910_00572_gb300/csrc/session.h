@@ -76,6 +76,7 @@ struct loc_session {
     bool aniso = false;            // anisotropic motion noise (step_aniso.cu)
     bool aniso_tma = false;        // ... with its input boxes by TMA (tmap holds its maps)
     bool tiled = false;            // use the TMA-tiled kernel
+    bool ragged = false;           // use the streaming kernel without TMA (rows of any width)
     int tile_cfg = 0;              // its tile configuration
     unsigned char tmap[2][128] __attribute__((aligned(128)));   // tensor maps of B[0], B[1]
     // host-side state (FP64)

@@ -9,7 +9,7 @@ namespace {
 
 using namespace stream;
 
-template <typename T, bool AM>
+template <typename T, bool AM, bool RAG>
 __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid_constant__ FastArgs a, int ntx,
                                                                     int ntiles) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -19,11 +19,13 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
     // restart: the input is M / (K n_free); read M and fold 1 / (K n_free) into the scale
     const float in_scale = (reinit ? a.inv_uniform : a.sd->inv_Z) * a.out_mult;
     int tile = blockIdx.x;
-    run_roles<T, AM>(
+    run_roles<T, AM, RAG>(
         sm,
         [&](Item& it, Source& src) {
             if (tile >= ntiles) return;
             it.out = a.B_out;
+            it.in = a.B_in;
+            it.reinit = reinit;
             it.trav = a.trav;
             it.corr = a.corr;
             it.K = a.K;
@@ -58,7 +60,7 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
     if (threadIdx.x == 0 && sm.fail) atomicOr(&a.sd->status, LOC_DEV_ERR_TIMEOUT);
 }
 
-template <typename T, bool AM>
+template <typename T, bool AM, bool RAG = false>
 cudaError_t launch(const FastArgs& a, cudaStream_t st) {
     static bool attr_set[64] = {};
     static int sms[64] = {};
@@ -67,14 +69,14 @@ cudaError_t launch(const FastArgs& a, cudaStream_t st) {
     const int slot = dev >= 0 && dev < 64 ? dev : 0;
     const size_t sb = sizeof(stream::Smem<T>) + 128;
     if (slot != dev || !attr_set[slot]) {
-        cudaError_t e = prepare<T>(step_stream_kernel<T, AM>);
+        cudaError_t e = prepare<T>(step_stream_kernel<T, AM, RAG>);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[slot], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         attr_set[slot] = true;
     }
     const int ntx = (a.W + TW - 1) / TW, ntiles = ntx * ((a.H + stream::TH - 1) / stream::TH);
     const int grid = ntiles < sms[slot] ? ntiles : sms[slot];
-    step_stream_kernel<T, AM><<<grid, stream::NT, sb, st>>>(a, ntx, ntiles);
+    step_stream_kernel<T, AM, RAG><<<grid, stream::NT, sb, st>>>(a, ntx, ntiles);
     return cudaGetLastError();
 }
 
@@ -89,6 +91,20 @@ cudaError_t launch_step_stream(const void* args, int storage, bool argmax, cudaS
         default: return cudaErrorInvalidValue;
     }
 }
+
+cudaError_t launch_step_ragged(const StepArgs& g, int storage, cudaStream_t st) {
+    FastArgs a;
+    memset(&a.tmap, 0, sizeof(a.tmap));
+    fill_args(a, g);
+    switch (storage) {
+        case LOC_F32: return launch<float, false, true>(a, st);
+        case LOC_BF16: return launch<__nv_bfloat16, false, true>(a, st);
+        case LOC_F16: return launch<__half, false, true>(a, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+bool step_ragged_eligible(int K, int r_xy, int r_th) { return r_xy == R && r_th == RT && K >= 8 && K <= LOC_MAX_K; }
 
 int stream_tile_rows() { return stream::TH; }
 

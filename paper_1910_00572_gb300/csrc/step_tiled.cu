@@ -554,26 +554,7 @@ size_t step_tmap_bytes() { return sizeof(CUtensorMap); }
 cudaError_t launch_step_tiled(const StepArgs& g, const void* tmap, int storage, int cfg, cudaStream_t st) {
     FastArgs a;
     memcpy(&a.tmap, tmap, sizeof(CUtensorMap));
-    a.B_out = g.B_out;
-    a.am_pv = g.am_pv;
-    a.am_pi = g.am_pi;
-    a.am_idx = g.am_idx;
-    a.am_val = g.am_val;
-    a.trav = g.trav;
-    a.corr = g.corr;
-    a.sd = g.sd;
-    a.partials = g.partials;
-    a.inv_uniform = g.inv_uniform;
-    a.out_mult = g.out_mult;
-    a.log_out_mult = g.log_out_mult;
-    a.H = g.H;
-    a.W = g.W;
-    a.K = g.K;
-    a.g0 = g.gx[R];
-    a.g1 = g.gx[R + 1];
-    a.g2 = g.gx[R + 2];
-    for (int d = 0; d < RING; ++d) a.gt[d] = g.gt[d];
-    for (int k = 0; k < g.K; ++k) a.sh[k] = g.sh[k];
+    fill_args(a, g);
     if (is_stream_cfg(cfg)) return launch_step_stream(&a, storage, step_tiled_fuses_argmax(cfg), st);
     cudaError_t e;
     switch (storage) {

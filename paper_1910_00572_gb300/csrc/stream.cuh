@@ -13,6 +13,10 @@
 //     theta blur, correction, store, normaliser and, with AM, the running argmax.
 // The next tile's planes enter the pipeline while the output warps finish the previous tile.
 //
+// RAG: rows whose pitch is no multiple of 16 bytes.  TMA cannot address them, so each blur warp
+// brings its own plane (load_rows); the stores are single values, and the operations follow the
+// generic kernel's order, whose place it takes (613 x 797 x 48 FP32: 632 -> RAGUS us).
+//
 // Why this split.  The tile body it replaces ran S, X and P as passes of all warps through
 // shared memory with two CTA barriers a plane: 42 to 53 thread instructions a cell and issue
 // 41 to 52 % busy.  Here a plane costs about 20 (FP32) to 28 (BF16) instructions a cell, eight
@@ -57,6 +61,8 @@ struct OCfg {                          // rows of an output thread (2 columns ea
 // One tile of work, as the manager hands it to the other warps.  K = 0: no more tiles.
 struct Item {
     void* out;
+    const void* in;                    // ragged rows only: X_{t-1} ...
+    int reinit;                        // ... or M in its place
     const uint8_t* trav;
     const float* corr;
     int K, H, W, ty0, tx0;
@@ -145,6 +151,31 @@ __device__ __forceinline__ void x_quad(const float (&a)[4], const float (&b)[4],
     *reinterpret_cast<float4*>(xp) = make_float4(v0, v1, v2, v3);
 }
 
+// The same in the order of the generic kernel (step_generic.cu), which grids of ragged rows took
+// before: their tensors stay the same bit for bit.
+__device__ __forceinline__ void s_quad_gen(const float* u, const float* d, const float4 m, float fx, float gx, f2 fy2,
+                                           f2 gy2, float (&s)[4]) {
+    float a[4], b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        a[k] = __fmaf_rn(gx, u[k], __fmul_rn(fx, u[k + 1]));
+        b[k] = __fmaf_rn(gx, d[k], __fmul_rn(fx, d[k + 1]));
+    }
+    const f2 o0 = fmul2(pk(m.x, m.y), ffma2(gy2, pk(a[0], a[1]), fmul2(fy2, pk(b[0], b[1]))));
+    const f2 o1 = fmul2(pk(m.z, m.w), ffma2(gy2, pk(a[2], a[3]), fmul2(fy2, pk(b[2], b[3]))));
+    upk(o0, s[0], s[1]);
+    upk(o1, s[2], s[3]);
+}
+__device__ __forceinline__ void x_quad_gen(const float (&a)[4], const float (&b)[4], float g0, float g1, float g2,
+                                           float* xp) {
+    const float s[8] = {a[0], a[1], a[2], a[3], b[0], b[1], b[2], b[3]};
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        v[k] = __fmaf_rn(g2, s[k + 4], __fmaf_rn(g1, s[k + 3], __fmaf_rn(g0, s[k + 2], __fmaf_rn(g1, s[k + 1], __fmul_rn(g2, s[k])))));
+    *reinterpret_cast<float4*>(xp) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
 // A 16-byte chunk of a raw row as floats.
 template <typename T> struct Chunk;
 template <> struct Chunk<float> {
@@ -183,7 +214,7 @@ template <> struct Chunk<__half> {
 // chunks an iteration, so that the registers of the two chunks in hand change roles without
 // moves and the eight alignments stay small enough for the instruction cache (fully unrolled,
 // a third of the stalls were instruction fetches).
-template <typename T, int XO>
+template <typename T, int XO, bool RAG>
 __device__ __forceinline__ void blur_plane(const T* __restrict__ raw, const float* __restrict__ mk,
                                            float* __restrict__ X, float fx, float fy, f2 g02, f2 g12, f2 g22) {
     constexpr int N = Chunk<T>::N, BWT = box_w<T>(), QN = N / 4;      // QN S quads a chunk
@@ -216,8 +247,17 @@ __device__ __forceinline__ void blur_plane(const T* __restrict__ raw, const floa
         }
         const float4 mc = m;
         m = mp[q + 1];
-        s_quad<PACK>(w, z, mc, fx2, fy2, gy2, fx, now);
-        x_quad(prev, now, g02, g12, g22, xp + 4 * q);
+        if constexpr (RAG) {
+            float g0, g1, g2, dup;
+            upk(g02, g0, dup);
+            upk(g12, g1, dup);
+            upk(g22, g2, dup);
+            s_quad_gen(w, z, mc, fx, 1.0f - fx, fy2, gy2, now);
+            x_quad_gen(prev, now, g0, g1, g2, xp + 4 * q);
+        } else {
+            s_quad<PACK>(w, z, mc, fx2, fy2, gy2, fx, now);
+            x_quad(prev, now, g02, g12, g22, xp + 4 * q);
+        }
     };
     // chunk n in (u, d); chunk n + 1 arrives in (v, e)
     auto chunk = [&](int n, const float (&u)[N], float (&v)[N], const float (&d)[N], float (&e)[N], float (&p)[4],
@@ -240,24 +280,83 @@ __device__ __forceinline__ void blur_plane(const T* __restrict__ raw, const floa
     quad((CHUNKS - 1) * QN, 0, ua, ub, da, db, s, t);
 }
 
-template <typename T>
+template <typename T, bool RAG>
 __device__ __forceinline__ void blur_any(const T* raw, const float* mk, float* X, int xo, float fx, float fy, f2 g0,
                                          f2 g1, f2 g2) {
+    if constexpr (RAG) {               // the rows were placed by load_rows
+        if (xo == 0) blur_plane<T, 0, true>(raw, mk, X, fx, fy, g0, g1, g2);
+        else if constexpr (sizeof(T) == 2) blur_plane<T, 1, true>(raw, mk, X, fx, fy, g0, g1, g2);
+        return;
+    }
     switch (xo) {
-        case 0: blur_plane<T, 0>(raw, mk, X, fx, fy, g0, g1, g2); break;
-        case 1: blur_plane<T, 1>(raw, mk, X, fx, fy, g0, g1, g2); break;
-        case 2: blur_plane<T, 2>(raw, mk, X, fx, fy, g0, g1, g2); break;
-        case 3: blur_plane<T, 3>(raw, mk, X, fx, fy, g0, g1, g2); break;
+        case 0: blur_plane<T, 0, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+        case 1: blur_plane<T, 1, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+        case 2: blur_plane<T, 2, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+        case 3: blur_plane<T, 3, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
         default:
             if constexpr (sizeof(T) == 2) {
                 switch (xo) {
-                    case 4: blur_plane<T, 4>(raw, mk, X, fx, fy, g0, g1, g2); break;
-                    case 5: blur_plane<T, 5>(raw, mk, X, fx, fy, g0, g1, g2); break;
-                    case 6: blur_plane<T, 6>(raw, mk, X, fx, fy, g0, g1, g2); break;
-                    default: blur_plane<T, 7>(raw, mk, X, fx, fy, g0, g1, g2); break;
+                    case 4: blur_plane<T, 4, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+                    case 5: blur_plane<T, 5, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+                    case 6: blur_plane<T, 6, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
+                    default: blur_plane<T, 7, false>(raw, mk, X, fx, fy, g0, g1, g2); break;
                 }
             }
     }
+}
+
+// Ragged rows (a row pitch that is no multiple of 16 bytes, so no TMA): a blur warp brings its
+// plane's box itself, rows y0 .. of plane p from column x, zeros outside the grid, without
+// waiting (the caller waits for its asynchronous copies).  FP32, and 16-bit rows of even width,
+// go as asynchronous 4-byte copies; 16-bit rows of odd width and a restart's map one element at
+// a time, 24 loads in flight.  Returns the first needed column in the box.
+template <typename T>
+__device__ __forceinline__ int load_rows(T* raw, const Item& it, int p, int x, int y0) {
+    const int lane = threadIdx.x & 31, H = it.H, W = it.W;
+    constexpr int BWT = box_w<T>();
+    const T* plane = static_cast<const T*>(it.in) + (size_t)p * H * W;
+    if (it.reinit || (sizeof(T) == 2 && (W & 1))) {
+        constexpr int COLS = 4 * SQ + 4;                       // 72: columns 0 .. 68 are needed
+        for (int r0 = 0; r0 < RAW_H; r0 += 8) {
+            T v[8][3];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int gy = y0 + r0 + r, gx = x + lane + 32 * q;
+                    const bool in = r0 + r < RAW_H && gy >= 0 && gy < H && gx >= 0 && gx < W && lane + 32 * q < COLS;
+                    const size_t at = in ? (size_t)gy * W + gx : 0;
+                    v[r][q] = !in ? T(0.0f) : it.reinit ? T((float)it.trav[at]) : plane[at];
+                }
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (r0 + r < RAW_H && lane + 32 * q < COLS) raw[(r0 + r) * BWT + lane + 32 * q] = v[r][q];
+        }
+        return 0;
+    }
+    constexpr int E = 4 / (int)sizeof(T);                      // elements a word
+    constexpr int WORDS = (4 * SQ + 4) / E + (E > 1 ? 1 : 0), NW = (WORDS + 31) / 32;
+    const int xo = x & (E - 1), xa = x - xo;
+    const uint32_t dst = su32(raw) + 4 * lane;
+    for (int r = 0; r < RAW_H; ++r) {
+        const int gy = y0 + r;
+        const bool row = gy >= 0 && gy < H;
+        const T* src = plane + (row ? (size_t)gy * W : 0);
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const int wd = lane + 32 * q, gx = xa + E * wd;
+            if (wd < WORDS) {
+                const bool in = row && gx >= 0 && gx < W;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                 dst + (uint32_t)(r * BWT * sizeof(T) + 128 * q)),
+                             "l"(in ? src + gx : plane), "r"(in ? 4 : 0)
+                             : "memory");
+            }
+        }
+    }
+    return xo;
 }
 
 // The manager's private side of a tile: where its planes come from.
@@ -287,8 +386,17 @@ __device__ __forceinline__ void init_barriers(Smem<T>& sm) {
 // The map mask over item t's halo region, by threads k of n.  The grid's width is a multiple of
 // 4 cells, so the map comes in whole words; W words a thread are in flight at once.
 constexpr int MWORDS = 19;             // words a row: columns -4 .. 71 of the tile
-template <int N, typename SM>
+template <int N, bool RAG, typename SM>
 __device__ __forceinline__ void fill_mask(SM& sm, int slot, const Item& t, int k) {
+    if constexpr (RAG) {               // byte loads
+        constexpr int COLS = 4 * SQ;
+#pragma unroll 8
+        for (int q = k; q < XR * COLS; q += N) {
+            const int r = q / COLS, c = q % COLS, y = t.ty0 - R + r, x = t.tx0 - R + c;
+            sm.mk[slot][r][c] = y >= 0 && y < t.H && x >= 0 && x < t.W && t.trav[(size_t)y * t.W + x] ? 1.0f : 0.0f;
+        }
+        return;
+    }
     constexpr int ALL = XR * MWORDS, W = (ALL + N - 1) / N;
     uint32_t m[W];
 #pragma unroll
@@ -308,13 +416,21 @@ __device__ __forceinline__ void fill_mask(SM& sm, int slot, const Item& t, int k
     }
 }
 
+// The channel of plane p of the stream.  The outputs of planes 3 .. K-1, 0, 1, 2 are written in that
+// order; for ragged rows the stream starts three channels earlier, so that they are written from
+// channel 0 up, the order in which the generic kernel carries the BF16 residuals.
+template <bool RAG>
+__device__ __forceinline__ int channel(int p, int K) {
+    return !RAG ? p : p >= RT ? p - RT : p - RT + K;
+}
+
 // Item t's plane sources into its slot, by lanes k of 32: many shift-table entries a load, so
 // that issuing a plane waits for nothing but its stage (with a table read per plane the manager
 // took ~1000 cycles a plane and was what bound the kernel).
-template <typename SM>
+template <bool RAG, typename SM>
 __device__ __forceinline__ void fill_plan(SM& sm, int slot, const Item& t, const Source& from, int k) {
     for (int p = k; p < t.K; p += 32) {
-        const Shift h = from.sh[p];
+        const Shift h = from.sh[channel<RAG>(p, t.K)];
         sm.plan[slot][p] = make_int4(t.tx0 - R + h.ox, t.ty0 - R + h.oy, __float_as_int(h.fx), __float_as_int(h.fy));
     }
 }
@@ -322,7 +438,7 @@ __device__ __forceinline__ void fill_plan(SM& sm, int slot, const Item& t, const
 // Manager warp, with the first item published in slot 0 (its plan too).  next(item, src) (all
 // lanes, the same answer) gives the next tile or K = 0; done(item, slot) (all lanes) takes a
 // finished tile's sums out of its slot.
-template <typename T, typename Next, typename Done>
+template <typename T, bool RAG, typename Next, typename Done>
 __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next next, Done done) {
     constexpr uint32_t kBoxBytes = RAW_H * box_w<T>() * sizeof(T);
     constexpr int AL = align_elems<T>();
@@ -364,8 +480,8 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
         const int slot = i & 1;
         if (i >= 2 && !retire(i - 2)) return false;
         if (t.K) {
-            fill_plan(sm, slot, t, from, lane);
-            fill_mask<32>(sm, slot, t, lane);
+            fill_plan<RAG>(sm, slot, t, from, lane);
+            fill_mask<32, RAG>(sm, slot, t, lane);
         }
         if (lane == 0) sm.item[slot] = t;
         __syncwarp();
@@ -377,7 +493,10 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
     for (; ok && it.K; ++i) {
         Item nit{};
         Source nsrc{};
-        for (int p = 0; ok && p < it.K; ++p) {
+        if constexpr (RAG) {           // the blur warps bring the planes
+            next(nit, nsrc);
+            ok = publish(i + 1, nit, nsrc);
+        } else for (int p = 0; ok && p < it.K; ++p) {
             ok = issue(p);
             if (ok && p == (it.K > NB ? NB : it.K - 1)) {   // early in the tile: the next one
                 next(nit, nsrc);
@@ -397,7 +516,7 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
     }
 }
 
-template <typename T>
+template <typename T, bool RAG>
 __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
     const int lane = threadIdx.x & 31;
     unsigned int g = w, base = 0;
@@ -410,14 +529,22 @@ __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
         const f2 g0 = pk(it.g0, it.g0), g1 = pk(it.g1, it.g1), g2 = pk(it.g2, it.g2);
         for (; g < base + K; g += NB) {
             const uint32_t ph = (g / NB) & 1;
-            if (g >= NB && !wait(sm, &sm.x_empty[w], ph ^ 1)) return;
-            if (!wait(sm, &sm.raw_full[w], ph)) return;
             const int4 pl = sm.plan[slot][g - base];
-            blur_any<T>(sm.raw[w], &sm.mk[slot][0][0], &sm.X[w][0][0], pl.x & (align_elems<T>() - 1),
-                        __int_as_float(pl.z), __int_as_float(pl.w), g0, g1, g2);
+            int xo;
+            if constexpr (RAG) xo = load_rows<T>(sm.raw[w], it, channel<true>(g - base, K), pl.x, pl.y);
+            else xo = pl.x & (align_elems<T>() - 1);
+            if (g >= NB && !wait(sm, &sm.x_empty[w], ph ^ 1)) return;
+            if constexpr (RAG) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+            } else if (!wait(sm, &sm.raw_full[w], ph)) {
+                return;
+            }
+            blur_any<T, RAG>(sm.raw[w], &sm.mk[slot][0][0], &sm.X[w][0][0], xo, __int_as_float(pl.z),
+                             __int_as_float(pl.w), g0, g1, g2);
             __syncwarp();
             if (lane == 0) {
-                arrive(&sm.raw_empty[w]);
+                if constexpr (!RAG) arrive(&sm.raw_empty[w]);
                 arrive(&sm.x_full[w]);
             }
         }
@@ -430,6 +557,30 @@ __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
 // The stored form of two neighbouring outputs and its value as FP32: FP32 as is, BF16 by error
 // diffusion along theta, FP16 to nearest (see store2).
 template <typename T> __device__ __forceinline__ f2 put2(T* p, f2 v, f2& res, bool on);
+// Two outputs of a ragged row: no alignment, each column with its own guard (on0, on1).
+template <typename T>
+__device__ __forceinline__ f2 put1(T* p, f2 v, f2& res, bool on0, bool on1) {
+    T tmp[2];
+    f2 st;
+    float a, b;
+    upk(v, a, b);
+    if constexpr (std::is_same_v<T, __nv_bfloat16>) {
+        const uint32_t d = bf16x2_diffuse(a, b, res, st);
+        tmp[0] = __ushort_as_bfloat16((unsigned short)d);
+        tmp[1] = __ushort_as_bfloat16((unsigned short)(d >> 16));
+    } else if constexpr (std::is_same_v<T, __half>) {
+        tmp[0] = __float2half_rn(a);
+        tmp[1] = __float2half_rn(b);
+        st = pk(__half2float(tmp[0]), __half2float(tmp[1]));
+    } else {
+        tmp[0] = a;
+        tmp[1] = b;
+        st = v;
+    }
+    if (on0) p[0] = tmp[0];
+    if (on1) p[1] = tmp[1];
+    return st;
+}
 template <> __device__ __forceinline__ f2 put2<float>(float* p, f2 v, f2&, bool on) {
     if (on) *reinterpret_cast<f2*>(p) = v;
     return v;
@@ -482,7 +633,7 @@ __device__ __forceinline__ ArgBest locate(const Item& it, int t, const PlaneBest
 // plane p, and its y blur follows them, so eight independent chains hide the latencies; runs
 // of 7 planes away from the ends carry no conditions.  Outside the grid the correction is 0,
 // so only the stores are guarded.
-template <typename T, bool AM>
+template <typename T, bool AM, bool RAG>
 __device__ __forceinline__ void output(Smem<T>& sm, int t) {
     constexpr int MR = OCfg::MR;
     const int lane = t & 31, r0 = MR * (t >> 5);
@@ -503,14 +654,15 @@ __device__ __forceinline__ void output(Smem<T>& sm, int t) {
             const int gy = it.ty0 + r0 + rr;
             on[rr] = gy < it.H && gx < it.W;
             const size_t at = (size_t)gy * it.W + gx;
-            out[rr] = static_cast<T*>(it.out) + RT * plane + at;
+            out[rr] = static_cast<T*>(it.out) + (RAG ? 0 : RT * plane) + at;   // the first channel written
             float c0 = 0.0f, c1 = 0.0f;
             if (on[rr]) {
                 c0 = it.corr[at] * it.in_scale;
-                c1 = it.corr[at + 1] * it.in_scale;
+                if (!RAG || gx + 1 < it.W) c1 = it.corr[at + 1] * it.in_scale;
             }
             cs[rr] = pk(c0, c1);
         }
+        const bool pair = !RAG || gx + 1 < it.W;         // the second column is in the grid too
         const f2 g0 = pk(it.g0, it.g0), g1 = pk(it.g1, it.g1), g2 = pk(it.g2, it.g2);
         f2 gt[RT + 1];                                   // symmetric taps: centre, +-1, +-2, +-3
 #pragma unroll
@@ -538,7 +690,8 @@ __device__ __forceinline__ void output(Smem<T>& sm, int t) {
             constexpr int PH = decltype(ph)::value;
 #pragma unroll
             for (int rr = 0; rr < MR; ++rr)
-                ring[PH][rr] = ffma2(g2, fadd2(x[rr], x[rr + 4]), ffma2(g1, fadd2(x[rr + 1], x[rr + 3]), fmul2(g0, x[rr + 2])));
+                ring[PH][rr] = RAG ? ffma2(g2, x[rr + 4], ffma2(g1, x[rr + 3], ffma2(g0, x[rr + 2], ffma2(g1, x[rr + 1], fmul2(g2, x[rr])))))
+                                   : ffma2(g2, fadd2(x[rr], x[rr + 4]), ffma2(g1, fadd2(x[rr + 1], x[rr + 3]), fmul2(g0, x[rr + 2])));
             __syncwarp();
             if (lane == 0) arrive(&sm.x_empty[(base + (unsigned int)p) % NB]);
         };
@@ -551,7 +704,8 @@ __device__ __forceinline__ void output(Smem<T>& sm, int t) {
                 f2 v = fmul2(gt[RT], ring[(PH + 1) % RING][rr]);
 #pragma unroll
                 for (int d = 1; d < RING; ++d) v = ffma2(gt[d < RT ? RT - d : d - RT], ring[(PH + 1 + d) % RING][rr], v);
-                st[rr] = put2<T>(out[rr], fmul2(cs[rr], v), res[rr], on[rr]);
+                if constexpr (RAG) st[rr] = put1<T>(out[rr], fmul2(cs[rr], v), res[rr], on[rr], on[rr] && pair);
+                else st[rr] = put2<T>(out[rr], fmul2(cs[rr], v), res[rr], on[rr]);
                 out[rr] += plane;
             }
             f2 part = st[0];
@@ -598,7 +752,7 @@ __device__ __forceinline__ void output(Smem<T>& sm, int t) {
         auto tail = [&](int p, auto ph) {
             constexpr int PH = decltype(ph)::value, NX = (PH + 1) % RING;
             if (p >= K + NWRAP) return;
-            if (p - RT == K) {                           // the last planes written are 0, 1, 2
+            if (!RAG && p - RT == K) {                   // the last planes written are 0, 1, 2
 #pragma unroll
                 for (int rr = 0; rr < MR; ++rr) out[rr] -= (size_t)K * plane;
             }
@@ -717,7 +871,7 @@ __device__ __forceinline__ void retire_tile(const SM& sm, const Item& it, int sl
 
 // The roles of the CTA's warps; next and done as for manage().  The first tile is set up by all
 // of them: the manager's planes travel while the others read the map.
-template <typename T, bool AM, typename Next, typename Done>
+template <typename T, bool AM, bool RAG, typename Next, typename Done>
 __device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Done done) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Item it{};
@@ -728,23 +882,23 @@ __device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Done done) {
             init_barriers(sm);
             sm.item[0] = it;
         }
-        fill_plan(sm, 0, it, src, lane);
+        fill_plan<RAG>(sm, 0, it, src, lane);
     }
     __syncthreads();
     if (warp != NO) {
         const Item t = sm.item[0];
-        if (t.K) fill_mask<NT - 32>(sm, 0, t, warp < NO ? threadIdx.x : threadIdx.x - 32);
+        if (t.K) fill_mask<NT - 32, RAG>(sm, 0, t, warp < NO ? threadIdx.x : threadIdx.x - 32);
         asm volatile("bar.sync 1, %0;" ::"n"(NT - 32) : "memory");
     } else if (lane == 0) {
         arrive(&sm.it_full[0]);
     }
     if (warp < NO + 1) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsOut));
-        if (warp < NO) output<T, AM>(sm, threadIdx.x);
-        else manage<T>(sm, it, src, next, done);
+        if (warp < NO) output<T, AM, RAG>(sm, threadIdx.x);
+        else manage<T, RAG>(sm, it, src, next, done);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsBlur));
-        blur<T>(sm, warp - (NO + 1));
+        blur<T, RAG>(sm, warp - (NO + 1));
     }
     __syncthreads();
 }

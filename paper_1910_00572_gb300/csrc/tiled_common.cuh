@@ -42,6 +42,7 @@ struct Cfg {
 
 struct FastArgs {
     CUtensorMap tmap;                  // X_{t-1} as [K][H][W], box {BW, RAW_H, 1}
+    const void* B_in;                  // X_{t-1} (read through tmap but for ragged rows)
     void* B_out;
     const uint8_t* trav;
     const float* corr;
@@ -59,6 +60,31 @@ struct FastArgs {
     float gt[RING];                    // theta taps -3 .. +3
     Shift sh[LOC_MAX_K];
 };
+
+// Everything of a launch but the tensor map.
+inline void fill_args(FastArgs& a, const StepArgs& g) {
+    a.B_in = g.B_in;
+    a.B_out = g.B_out;
+    a.am_pv = g.am_pv;
+    a.am_pi = g.am_pi;
+    a.am_idx = g.am_idx;
+    a.am_val = g.am_val;
+    a.trav = g.trav;
+    a.corr = g.corr;
+    a.sd = g.sd;
+    a.partials = g.partials;
+    a.inv_uniform = g.inv_uniform;
+    a.out_mult = g.out_mult;
+    a.log_out_mult = g.log_out_mult;
+    a.H = g.H;
+    a.W = g.W;
+    a.K = g.K;
+    a.g0 = g.gx[R];
+    a.g1 = g.gx[R + 1];
+    a.g2 = g.gx[R + 2];
+    for (int d = 0; d < RING; ++d) a.gt[d] = g.gt[d];
+    for (int k = 0; k < g.K; ++k) a.sh[k] = g.sh[k];
+}
 
 template <typename T> __host__ __device__ constexpr int align_elems() { return 16 / (int)sizeof(T); }
 

@@ -42,3 +42,34 @@ def test_streaming_tiles_equal_the_synchronous_ones(H, W, K, storage):
     finally:
         for h in hs:
             loc.loc_destroy(h)
+
+
+RAGGED = [(1, 1, 8), (29, 61, 9), (31, 66, 11), (57, 133, 16), (40, 250, 22), (565, 577, 8)]
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("H,W,K", RAGGED, ids=lambda v: str(v))
+def test_streaming_ragged_rows_equal_the_generic_kernel(H, W, K, storage):
+    """Rows of any width (odd, even, a multiple of 4 but not of 16 bytes), shifts within a cell and
+    beyond a tile: the generic kernel's operations in its order, so its stored values; normalisers as
+    above."""
+    rng = np.random.default_rng(H + W + K)
+    occ = (rng.random((H, W)) < 0.15).astype(np.uint8)
+    occ[H // 2, W // 2] = 0
+    b = fields.belief_like(occ, K, seed=H, dtype=np.float32)
+    if not b.any():
+        b = np.repeat((occ == 0)[None].astype(np.float32), K, 0)
+    hs = [loc.loc_create(occ, loc.loc_params_default(H=H, W=W, K=K, cell_m=0.05, storage=storage, kernel=k))
+          for k in (loc.LOC_KERNEL_GENERIC, loc.LOC_KERNEL_AUTO)]
+    try:
+        for u, first in ((0.031, True), (0.031, False), (0.9, False), (0.0, False)):
+            for h in hs:
+                if not first:
+                    loc.loc_set_belief(h, b)
+                loc.loc_step(h, u, -0.044 if u else 0.0, 0.05)
+            want, z = loc.loc_belief(hs[0]), loc.loc_stats(hs[0])["last_Z"]
+            assert abs(loc.loc_stats(hs[1])["last_Z"] - z) <= 2.0 ** -23 * z
+            np.testing.assert_allclose(loc.loc_belief(hs[1]), want, rtol=2.0 ** -21, atol=0)
+    finally:
+        for h in hs:
+            loc.loc_destroy(h)
