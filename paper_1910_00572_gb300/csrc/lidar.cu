@@ -8,6 +8,9 @@
 #include <algorithm>
 #include <cfloat>
 
+#include <cooperative_groups.h>
+#include <type_traits>
+
 #include "dda.cuh"
 #include "kernels.h"
 
@@ -112,18 +115,20 @@ __global__ void __launch_bounds__(NT) belief_map_vec_kernel(const T* __restrict_
 // the whole map is a wavefront of W + 94 + (blocks - 1) x (94 + hand-off) steps.  One CTA of 16
 // warps (four rows of blocks one after the other, 16 warps on four schedulers, a fence per
 // hand-off) took 1.73 ms at 2048 x 2048; a warp per block on a scheduler of its own, with
-// hand-offs that need no fence, takes FSUS.  The cluster keeps the warps that wait on one another
-// resident together.
+// hand-offs that need no fence, takes 0.42 (66 cycles a step, ten thousand cycles from a block's
+// start to the next one's).  The cluster keeps the warps that wait on one another resident together.
 //
-// Hand-off: a block's last lane writes its errors to bnd[rb + 1][*] as it goes.  The whole buffer
-// starts as kFsEmpty (a NaN that no arithmetic produces), so a value that is not kFsEmpty is
-// there: the next block polls the 32 values of its window themselves, with a limit.
+// Hand-off: a block's last lane writes its errors into the next block's inbox as it goes: shared
+// memory of the next block's CTA, through the cluster (bnd in global memory where the rows are too
+// long for that: ~1000 cycles a hand-off, 0.82 ms at 2048 x 2048).  An inbox starts as kFsEmpty (a
+// NaN that no arithmetic produces), so a value that is not kFsEmpty is there and needs no fence: the
+// next block polls the kFsSub values it needs next, with a limit.
 //
-// Each warp keeps a ring of four 32-column chunks per row in shared memory (column i at position
-// i mod 128), the first chunk repeated behind the fourth so that a window of 32 steps reads at
-// constant offsets; a pitch of 162 makes the lanes' 3-column skew hit distinct banks.  At step
-// 32 T the last lane has finished chunk T - 4, so chunk T of the map (loaded into registers,
-// coalesced, one window earlier) takes its place.  Selections are bits: a lane collects a window's
+// A second warp per block brings the map: a ring of six 32-column chunks per row in shared memory
+// (column i at position i mod 192), the first chunk repeated behind the sixth so that a window of
+// 32 steps reads at constant offsets; a pitch of 226 makes the lanes' 3-column skew hit distinct
+// banks.  A window reads chunks T - 3 .. T, so the ring is two chunks ahead.  (Done by the block's
+// own warp between its windows, the copy took a third of the time.)  Selections are bits: a lane collects a window's
 // 32 and writes them as one aligned word of its row.  Terms of the error sum whose source lies
 // outside the grid are zero (their errors were never produced), so the sum always takes the same
 // four terms in the same order; only the right neighbour above is masked at the last column.
@@ -133,144 +138,205 @@ constexpr int kFsWarps = 4;               // one per scheduler
 constexpr int kFsMaxCtas = 16;            // largest cluster: 64 blocks of 32 rows side by side
 constexpr int kFsSkew = 3;
 constexpr int kFsLead = 32 * kFsSkew;     // steps of skew over a block, rounded up: 93 -> 96
-constexpr int kFsPitch = 162;
+constexpr int kFsChunks = 6, kFsRing = 32 * kFsChunks, kFsPitch = 226;
 constexpr uint32_t kFsEmpty = 0xFFFFFFFFu;
+constexpr int kFsSub = 16;                // steps between two looks at the inbox
+constexpr int kFsPad = kFsSub - 1;        // column c of an inbox lies at c + 15: looks are aligned
+constexpr size_t kFsRingBytes = sizeof(float) * kFsWarps * 32 * kFsPitch;
+constexpr size_t kFsInboxBytes = 108 * 1024;   // shared memory for the inboxes of a CTA at most
 
-__global__ void __launch_bounds__(kFsWarps * 32) fs_kernel(const float* __restrict__ m, const float* fs_ptr, int H,
+// inboxes a warp: two where it takes several blocks (the block above its next one may write while
+// it still reads), each W rounded up to a multiple of 32
+template <bool DSM>
+__global__ void __launch_bounds__(kFsWarps * 64) fs_kernel(const float* __restrict__ m, const float* fs_ptr, int H,
                                                            int W, uint32_t* __restrict__ selbits,
-                                                           int* __restrict__ rowcnt, float* bnd, int* status) {
-    extern __shared__ float fs_ring_all[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                                                           int* __restrict__ rowcnt, float* bnd, int nbox, int* status) {
+    extern __shared__ __align__(16) float fs_ring_all[];
+    __shared__ volatile int s_filled[kFsWarps], s_done[kFsWarps];   // chunks brought, windows done
+    namespace cg = cooperative_groups;
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % kFsWarps;
+    const bool loader = threadIdx.x >= kFsWarps * 32;
     float* ring = fs_ring_all + (size_t)warp * 32 * kFsPitch;
-    const float* own = ring + lane * kFsPitch;                 // this lane's row
-    const float fs = *fs_ptr;
     const unsigned long long wait_ns = g_fs_wait_ns;
     const int stall = g_fs_stall;
     const int nrb = (H + 31) / 32, nch = (W + 31) / 32;
+    const int nwin = (W + kFsSkew * 31 + 31) / 32;
     const float w7 = 0.4375f, w3 = 0.1875f, w5 = 0.3125f, w1 = 0.0625f;
-    for (int rb = blockIdx.x * kFsWarps + warp; rb < nrb; rb += gridDim.x * kFsWarps) {
+    const int wpad = 32 * nch + 64;
+    float* box_all = fs_ring_all + kFsRingBytes / sizeof(float);
+    auto inbox = [&](int w, int round) { return box_all + (size_t)(w * nbox + (nbox == 2 ? round & 1 : 0)) * wpad; };
+    if (threadIdx.x < kFsWarps) s_filled[threadIdx.x] = s_done[threadIdx.x] = 0;
+    if constexpr (DSM) {
+        for (int q = threadIdx.x; q < kFsWarps * nbox * wpad; q += kFsWarps * 64) box_all[q] = __uint_as_float(kFsEmpty);
+        cg::this_cluster().sync();
+    } else {
+        __syncthreads();
+    }
+    bool failed = false;
+    // a whole warp's wait with a limit; ready() gives every lane the same answer
+    auto await = [&](auto ready) {
+        if (ready()) return;
+        const unsigned long long g0 = gtime();
+        for (unsigned int it = 0; !ready();)
+            if (__any_sync(0xffffffffu, ++it > (1u << 24) || gtime() - g0 > wait_ns)) {
+                if (lane == 0) atomicOr(status, LOC_DEV_ERR_TIMEOUT);
+                failed = true;                                 // the blocks below run into their limits too
+                return;
+            }
+    };
+    int round = 0;
+    for (int rb = blockIdx.x * kFsWarps + warp; rb < nrb && !failed; rb += gridDim.x * kFsWarps, ++round) {
         const int j0 = 32 * rb, j = j0 + lane;
         const bool row_ok = j < H;
         const bool interior = j0 + 31 < H;                     // every row of the block in the grid
-        float pre[32];                                         // column 32 c + lane of rows j0 ..
-        auto load_chunk = [&](int c) {
-            const int col = 32 * c + lane;
-            if (interior && col < W) {
+        if (loader) {
+            const float fs = *fs_ptr;
+            float pre[32];                                     // column 32 c + lane of rows j0 ..
+            auto load_chunk = [&](int c) {
+                const int col = 32 * c + lane;
                 const float* src = m + (size_t)j0 * W + col;
 #pragma unroll
-                for (int r = 0; r < 32; ++r) pre[r] = __ldg(src + (size_t)r * W);
-            } else {
+                for (int r = 0; r < 32; ++r) pre[r] = (interior || j0 + r < H) && col < W ? __ldg(src + (size_t)r * W) : 0.0f;
+            };
+            load_chunk(0);
+            for (int c = 0; c < nch && !failed; ++c) {
+                // chunk c takes the place of chunk c - 6, last read in window c - 3; the first chunk
+                // waits for the end of the block before
+                const int need = round * nwin + (c >= kFsChunks - 3 ? c - (kFsChunks - 4) : 0);
+                await([&]() { return s_done[warp] >= need; });
+                __syncwarp();
+                float* dst = ring + (c % kFsChunks) * 32 + lane;
 #pragma unroll
-                for (int r = 0; r < 32; ++r)
-                    pre[r] = (j0 + r < H && col < W) ? __ldg(m + (size_t)(j0 + r) * W + col) : 0.0f;
+                for (int r = 0; r < 32; ++r) {
+                    float v = __fmul_rn(pre[r], fs);
+                    if (v > 1.0f) v = 1.0f;
+                    dst[r * kFsPitch] = v;
+                    if (c % kFsChunks == 0) dst[r * kFsPitch + kFsRing] = v;
+                }
+                __threadfence_block();
+                __syncwarp();
+                if (lane == 0) s_filled[warp] = round * nch + c + 1;
+                if (c + 1 < nch) load_chunk(c + 1);
             }
-        };
-        auto store_chunk = [&](int c) {
-            float* dst = ring + (c & 3) * 32 + lane;
-#pragma unroll
-            for (int r = 0; r < 32; ++r) {
-                float v = __fmul_rn(pre[r], fs);
-                if (v > 1.0f) v = 1.0f;
-                dst[r * kFsPitch] = v;
-                if ((c & 3) == 0) dst[r * kFsPitch + 128] = v;
-            }
-        };
-        __syncwarp();                                          // the previous block's reads are done
-        load_chunk(0);
-        store_chunk(0);
-        if (nch > 1) load_chunk(1);
-        __syncwarp();
+            continue;
+        }
+        const float* own = ring + lane * kFsPitch;             // this lane's row
         float up_old = 0.0f, up_mid = 0.0f, up_new = 0.0f;   // row above: columns i-1, i, i+1
         float pend = 0.0f;                                     // ... and the next one, for the next step
         float last = 0.0f;                                     // own error at the column before
-        float chunk = 0.0f;                                    // lane L: bnd[rb][t0 + 1 + L]
         uint32_t before = 0;                                   // the previous window's selections
         int cnt = 0;
         const int r_off = (kFsLead - kFsSkew * lane) & 31;     // (t0 - 3 lane) mod 32, t0 a multiple of 32
         const bool publish = lane == 31 && rb + 1 < nrb;       // the next block reads this row
-        float* bnd_next = bnd + (size_t)(rb + 1 < nrb ? rb + 1 : rb) * W;
-        const volatile uint32_t* above = reinterpret_cast<const volatile uint32_t*>(bnd) + (size_t)rb * W;
-        const int nwin = (W + kFsSkew * 31 + 31) / 32;
-        for (int T = 0; T < nwin; ++T) {
-            const int t0 = 32 * T;
-            if (rb > 0) {
-                // the row above, columns t0 + 1 .. t0 + 32 (and column 0 before the first step:
-                // lane 0 starts there at once; other lanes shift theirs in while they wait)
-                const int c = t0 + 1 + lane;
-                uint32_t v = 0u, v0 = 0u;
-                const unsigned long long g0 = gtime();
-                unsigned int it = 0;
-                bool ok;
-                for (;;) {
-                    if (c < W) v = above[c];
-                    if (T == 0) v0 = above[0];
-                    ok = !stall && v != kFsEmpty && v0 != kFsEmpty;
-                    if (__all_sync(0xffffffffu, ok)) break;
-                    if (__any_sync(0xffffffffu, ++it > (1u << 22) || gtime() - g0 > wait_ns)) {
-                        if (lane == 0) atomicOr(status, LOC_DEV_ERR_TIMEOUT);
-                        return;                                // the blocks below run into their limits too
-                    }
-                }
-                chunk = __uint_as_float(v);
-                if (T == 0 && lane == 0) up_new = __uint_as_float(v0);
-            }
-            if (T > 0 && T < nch) {
-                __syncwarp();                                  // chunk T - 4 is read
-                store_chunk(T);
-                __syncwarp();
-                if (T + 1 < nch) load_chunk(T + 1);
-            }
-            const float* ow = own + ((t0 - kFsSkew * lane) & 127);
-            uint32_t bits = 0;
-            if (interior && t0 >= kFsSkew * 31 && t0 + 31 <= W - 2) {
-                // every lane's column lies in [0, W - 2] for the whole window and every row of the
-                // block is in the grid: no guards.  The same operations in the same order as the
-                // general steps below (0 + x == x exactly, and chunk is 0 with no row above).
+        float* below;                                          // the next block's inbox, and this one's
+        const volatile uint32_t* above;
+        if constexpr (DSM) {
+            const int cta = blockIdx.x + (warp + 1) / kFsWarps, to = cta % gridDim.x;
+            below = cg::this_cluster().map_shared_rank(inbox((warp + 1) % kFsWarps, round + cta / gridDim.x), to) + kFsPad;
+            above = reinterpret_cast<const volatile uint32_t*>(inbox(warp, round) + kFsPad);
+        } else {
+            below = bnd + (size_t)(rb + 1 < nrb ? rb + 1 : rb) * W;
+            above = reinterpret_cast<const volatile uint32_t*>(bnd) + (size_t)rb * W;
+        }
+        // the row above at columns c0 .. c0 + 15, c0 = 1 mod 16 (0 past the last one), every lane the same
+        struct Above {
+            uint32_t v[kFsSub];
+        };
+        auto look = [&](int c0) {
+            Above e;
 #pragma unroll
-                for (int s = 0; s < 32; ++s) {
-                    const float from_above = __shfl_sync(0xffffffffu, chunk, s);
-                    up_old = up_mid;
-                    up_mid = up_new;
-                    up_new = lane == 0 ? from_above : pend;
-                    pend = __shfl_up_sync(0xffffffffu, last, 1);
-                    const float v = ow[s];
-                    float E = __fmul_rn(up_old, w1);
-                    E = __fadd_rn(E, __fmul_rn(up_mid, w5));
-                    E = __fadd_rn(E, __fmul_rn(up_new, w3));
-                    E = __fadd_rn(E, __fmul_rn(last, w7));
-                    float val = __fadd_rn(v, E);
-                    if (val >= 0.5f) {
-                        val = __fsub_rn(val, 1.0f);
-                        bits |= 1u << s;
+            for (int k = 0; k < kFsSub; ++k) e.v[k] = 0u;
+            if (rb > 0 && c0 < W) {                            // (an inbox is padded past its last column)
+                if constexpr (DSM) {
+#pragma unroll
+                    for (int h = 0; h < kFsSub / 4; ++h) {
+                        uint32_t* v = e.v + 4 * h;
+                        asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                     : "r"((uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(above) + c0 + 4 * h)));
                     }
-                    last = val;
-                    if (publish) *reinterpret_cast<volatile float*>(bnd_next + t0 + s - kFsSkew * 31) = val;
-                }
-            } else {
-#pragma unroll 4
-                for (int s = 0; s < 32; ++s) {
-                    const float from_above = __shfl_sync(0xffffffffu, chunk, s);
-                    up_old = up_mid;
-                    up_mid = up_new;
-                    up_new = lane == 0 ? (rb > 0 ? from_above : 0.0f) : pend;
-                    pend = __shfl_up_sync(0xffffffffu, last, 1);
-                    const int i = t0 + s - kFsSkew * lane;
-                    const float v = ow[s];
-                    if ((unsigned)i < (unsigned)W && row_ok) {
-                        float E = __fadd_rn(0.0f, __fmul_rn(up_old, w1));
-                        E = __fadd_rn(E, __fmul_rn(up_mid, w5));
-                        E = __fadd_rn(E, __fmul_rn(i + 1 < W ? up_new : 0.0f, w3));
-                        E = __fadd_rn(E, __fmul_rn(last, w7));
-                        float val = __fadd_rn(v, E);
-                        if (val >= 0.5f) {
-                            val = __fsub_rn(val, 1.0f);
-                            bits |= 1u << s;
-                        }
-                        last = val;
-                        if (publish) *reinterpret_cast<volatile float*>(bnd_next + i) = val;
-                    }
+#pragma unroll
+                    for (int k = 0; k < kFsSub; ++k)
+                        if (c0 + k >= W) e.v[k] = 0u;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < kFsSub; ++k)
+                        if (c0 + k < W) e.v[k] = above[c0 + k];
                 }
             }
+            return e;
+        };
+        auto there = [&](const Above& e) {
+            uint32_t most = 0;                                 // kFsEmpty is the largest word
+#pragma unroll
+            for (int k = 0; k < kFsSub; ++k) most = max(most, e.v[k]);
+            return __all_sync(0xffffffffu, most != kFsEmpty && !(stall && rb > 0)) != 0;
+        };
+        // lane 0 starts at column 0 at once: the row above at column 0 must already be in its register
+        // chain (other lanes shift theirs in while they wait to start)
+        if (rb > 0) {
+            uint32_t v = kFsEmpty;
+            await([&]() {
+                v = above[0];
+                return __all_sync(0xffffffffu, !stall && v != kFsEmpty) != 0;
+            });
+            if (lane == 0) up_new = __uint_as_float(v);
+        }
+        Above next = look(1);
+        int at = (kFsRing - kFsSkew * lane) % kFsRing;         // ring position of the lane's column at t0
+        for (int T = 0; T < nwin && !failed; ++T) {
+            const int t0 = 32 * T, have = round * nch + (T < nch ? T : nch - 1);
+            await([&]() { return s_filled[warp] > have; });
+            __syncwarp();
+            const float* ow = own + at;
+            uint32_t bits = 0;
+            const bool plain = interior && t0 >= kFsSkew * 31 && t0 + 31 <= W - 2;
+#pragma unroll
+            for (int u = 0; u < 32; u += kFsSub) {
+                Above now = next;
+                if (!there(now)) await([&]() {
+                    now = look(t0 + u + 1);
+                    return there(now);
+                });
+                if (failed) break;
+                next = look(t0 + u + 1 + kFsSub);
+                float v[kFsSub];
+#pragma unroll
+                for (int k = 0; k < kFsSub; ++k) v[k] = ow[u + k];
+                // In a plain window every lane's column lies in [0, W - 2] and every row of the block is in
+                // the grid: no guards.  The others keep a lane's error as it is while its column is off the
+                // grid (0 before the first one) and mask the right neighbour above at the last column; the
+                // same operations in the same order (0 + x == x exactly).
+                auto steps = [&](auto guarded) {
+                    constexpr bool G = decltype(guarded)::value;
+#pragma unroll
+                    for (int k = 0; k < kFsSub; ++k) {
+                        const int i = t0 + u + k - kFsSkew * lane;
+                        up_old = up_mid;
+                        up_mid = up_new;
+                        up_new = lane == 0 ? __uint_as_float(now.v[k]) : pend;
+                        pend = __shfl_up_sync(0xffffffffu, last, 1);
+                        const bool in = !G || (row_ok && (unsigned)i < (unsigned)W);
+                        float E = __fmul_rn(up_old, w1);
+                        E = __fadd_rn(E, __fmul_rn(up_mid, w5));
+                        E = __fadd_rn(E, __fmul_rn(G && i + 1 >= W ? 0.0f : up_new, w3));
+                        E = __fadd_rn(E, __fmul_rn(last, w7));
+                        const float val = __fadd_rn(v[k], E), less = __fsub_rn(val, 1.0f);
+                        const bool on = val >= 0.5f;
+                        const float err = on ? less : val;
+                        last = in ? err : last;
+                        bits |= on && in ? 1u << (u + k) : 0u;
+                        if (publish && in) *reinterpret_cast<volatile float*>(below + i) = err;
+                    }
+                };
+                if (plain) steps(std::false_type{});
+                else steps(std::true_type{});
+            }
+            if (failed) break;
+            __syncwarp();
+            if (lane == 0) s_done[warp] = round * nwin + T + 1;
+            at += 32;
+            if (at >= kFsRing) at -= kFsRing;
             // the aligned word that this window completes: columns t0 - 3 lane - r_off ..
             const int c = (t0 - kFsSkew * lane - r_off) >> 5;
             const uint32_t word = __funnelshift_l(before, bits, r_off);
@@ -280,6 +346,7 @@ __global__ void __launch_bounds__(kFsWarps * 32) fs_kernel(const float* __restri
                 cnt += __popc(word);
             }
         }
+        if (failed) break;
         // the word that a lane's last window began, where it lies in the grid
         const int c = (32 * nwin - kFsSkew * lane - r_off) >> 5;
         if (row_ok && r_off > 0 && c >= 0 && c < nch) {
@@ -288,7 +355,17 @@ __global__ void __launch_bounds__(kFsWarps * 32) fs_kernel(const float* __restri
             cnt += __popc(word);
         }
         if (row_ok) rowcnt[j] = cnt;
+        if constexpr (DSM) {                                   // empty again for the block after next
+            if (nbox == 2) {
+                float* box = inbox(warp, round);
+                for (int q = lane; q < wpad; q += 32) box[q] = __uint_as_float(kFsEmpty);
+                __threadfence();
+                __syncwarp();
+            }
+        }
     }
+    // no CTA leaves while another may still write to its inboxes
+    if constexpr (DSM) cg::this_cluster().sync();
 }
 
 // Exclusive prefix of the per-row counts (one CTA); total -> *count.
@@ -609,23 +686,47 @@ cudaError_t launch_belief_map(const void* B, int storage, const uint8_t* trav, S
 cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_t* selbits, int* rowcnt, int* rowoff,
                           int* count, float* bnd, int* status, int cap, int32_t* samples, cudaStream_t st) {
     const int nrb = (H + 31) / 32;
-    cudaError_t e = cudaMemsetAsync(bnd, 0xFF, sizeof(float) * (size_t)nrb * W, st);   // kFsEmpty
-    if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(float) * kFsWarps * 32 * kFsPitch;
-    static bool attr_set[64] = {};
+    static int max_ctas[64] = {};                              // per device: the largest cluster it can hold
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(fs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fs_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const int slot = dev >= 0 && dev < 64 ? dev : 0;
+    cudaError_t e = cudaSuccess;
+    if (slot != dev || !max_ctas[slot]) {
+        const int most = (int)(kFsRingBytes + kFsInboxBytes);
+        for (auto* f : {fs_kernel<true>, fs_kernel<false>}) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        }
         if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+        int n = kFsMaxCtas, fit = 0;
+        for (; n > 1; n /= 2) {
+            cudaLaunchConfig_t q{};
+            cudaLaunchAttribute qa{};
+            qa.id = cudaLaunchAttributeClusterDimension;
+            qa.val.clusterDim.x = n;
+            qa.val.clusterDim.y = qa.val.clusterDim.z = 1;
+            q.gridDim = dim3(n);
+            q.blockDim = dim3(kFsWarps * 64);
+            q.dynamicSmemBytes = most;
+            q.attrs = &qa;
+            q.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&fit, fs_kernel<true>, &q) == cudaSuccess && fit > 0) break;
+            cudaGetLastError();
+        }
+        max_ctas[slot] = n;
     }
     int ctas = 1;                                              // a power of two, one warp per block
-    while (ctas < kFsMaxCtas && ctas * kFsWarps < nrb) ctas *= 2;
+    while (ctas < max_ctas[slot] && ctas * kFsWarps < nrb) ctas *= 2;
+    // the inboxes in shared memory where the rows fit
+    const int nbox = ctas * kFsWarps < nrb ? 2 : 1;
+    const size_t boxes = sizeof(float) * kFsWarps * nbox * (size_t)((W + 31) / 32 * 32 + 64);
+    const bool dsm = boxes <= kFsInboxBytes;
+    const size_t smem = kFsRingBytes + (dsm ? boxes : 0);
+    if (!dsm) e = cudaMemsetAsync(bnd, 0xFF, sizeof(float) * (size_t)nrb * W, st);   // kFsEmpty
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(kFsWarps * 32);
+    cfg.blockDim = dim3(kFsWarps * 64);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -634,7 +735,7 @@ cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, fs_kernel, m, fs, H, W, selbits, rowcnt, bnd, status);
+    e = cudaLaunchKernelEx(&cfg, dsm ? fs_kernel<true> : fs_kernel<false>, m, fs, H, W, selbits, rowcnt, bnd, nbox, status);
     if (e != cudaSuccess) return e;
     row_scan_kernel<<<1, 1024, 0, st>>>(rowcnt, H, rowoff, count, status);
     if (samples)

@@ -15,7 +15,7 @@
 //
 // RAG: rows whose pitch is no multiple of 16 bytes.  TMA cannot address them, so each blur warp
 // brings its own plane (load_rows); the stores are single values, and the operations follow the
-// generic kernel's order, whose place it takes (613 x 797 x 48 FP32: 632 -> RAGUS us).
+// generic kernel's order, whose place it takes (613 x 797 x 48 FP32: 634 -> 84 us).
 //
 // Why this split.  The tile body it replaces ran S, X and P as passes of all warps through
 // shared memory with two CTA barriers a plane: 42 to 53 thread instructions a cell and issue
