@@ -103,16 +103,17 @@ loc_status check_live(loc_session* h) {
 }
 
 loc_status sync_and_check(loc_session* h) {
-    cudaError_t e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamSynchronize");
-    // the device status and the restart count are adjacent in SessionDev: one copy
+    // the device status and the restart count are adjacent in SessionDev: one copy, through pinned
+    // memory, so that one wait covers it and the work before it
     struct {
         int status, pad;
         unsigned long long n_reinit;
     } d{};
     static_assert(offsetof(SessionDev, n_reinit) == offsetof(SessionDev, status) + 8, "SessionDev layout");
-    e = cudaMemcpy(&d, &h->sd->status, sizeof(d), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemcpy(status)");
+    cudaError_t e = cudaMemcpyAsync(h->pinned + 48, &h->sd->status, sizeof(d), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamSynchronize");
+    std::memcpy(&d, h->pinned + 48, sizeof(d));
     const loc_status st = check_status(h, d.status);
     if (st != LOC_OK) return st;
     if (d.n_reinit > h->reinit_reported) {         // restarts since the last report
@@ -959,6 +960,13 @@ LOC_API loc_status loc_map_difficulty(loc_handle h, const int32_t* probes, int n
     return sync_and_check(h);
 }
 
+// The session's H * W floats of readback scratch, allocated on first use (all its uses are on the
+// session's stream).
+static bool map_buffer(loc_session* h) {
+    if (!h->map_buf) h->map_buf = (float*)dev_alloc(h, h->hw * sizeof(float));
+    return h->map_buf != nullptr;
+}
+
 LOC_API loc_status loc_belief(loc_handle h, float* out, size_t n) {
     loc_status st = check_live(h);
     if (st != LOC_OK) return st;
@@ -980,14 +988,10 @@ LOC_API loc_status loc_marginal(loc_handle h, float* out, size_t n, int mode) {
     if (st != LOC_OK) return st;
     if (!out || n != h->hw) return fail(h, LOC_ERR_INVALID_ARG, "out null or n != H*W");
     if (mode != LOC_MAP_SUM && mode != LOC_MAP_MAX) return fail(h, LOC_ERR_INVALID_ARG, "mode");
-    float* tmp = (float*)dev_alloc(h, n * sizeof(float));
-    if (!tmp) return fail(h, LOC_ERR_OOM, "readback buffer");
+    if (!map_buffer(h)) return fail(h, LOC_ERR_OOM, "readback buffer");
     cudaError_t e = launch_read_marginal(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform,
-                                         h->p.H, h->p.W, h->p.K, mode, tmp, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->owned.pop_back();
-    if (g_free) g_free(tmp, (void*)h->stream, g_alloc_ctx); else cudaFree(tmp);
+                                         h->p.H, h->p.W, h->p.K, mode, h->map_buf, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, h->map_buf, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_marginal");
     return sync_and_check(h);
 }
@@ -1041,15 +1045,14 @@ LOC_API loc_status loc_estimate(loc_handle h, double radius_m, int dk, loc_estim
         h->est = (EstimateOut*)dev_alloc(h, sizeof(EstimateOut));
         if (!h->est) return fail(h, LOC_ERR_OOM, "estimate buffer");
     }
+    if (!map_buffer(h)) return fail(h, LOC_ERR_OOM, "estimate buffer");
     const double c = h->p.cell_m;
     // cells whose centres lie within radius_m; the 1e-9 keeps a whole number of cells inclusive
     const double r2d = std::floor(radius_m * radius_m / (c * c) + 1e-9);
     const long long r2 = r2d > 4.0e18 ? (long long)4e18 : (long long)r2d;
-    cudaError_t e = launch_argmax(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform, h->p.H, h->p.W, h->p.K,
-                                  h->argmax_scratch, h->argmax_idx, h->argmax_val, h->stream);
-    if (e == cudaSuccess)
-        e = launch_estimate(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform, h->p.H, h->p.W, h->p.K,
-                            h->argmax_scratch, h->argmax_idx, r2, dk, h->partials, h->nparts, h->est, h->stream);
+    cudaError_t e = launch_estimate(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform, h->p.H, h->p.W, h->p.K,
+                                    h->map_buf, h->argmax_scratch, h->argmax_idx, h->argmax_val, r2, dk, h->partials,
+                                    h->nparts, h->est, h->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->pinned, h->argmax_idx, sizeof(long long) + sizeof(float), cudaMemcpyDeviceToHost,
                             h->stream);

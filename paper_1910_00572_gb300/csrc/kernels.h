@@ -138,11 +138,12 @@ struct EstimateOut {
     float second_p;
     float pad;
 };
-// After launch_argmax on the same stream (its index in arg_idx; its scratch reused).
+// The argmax state (to arg_idx / arg_val, as launch_argmax) and the results around it; map: H * W
+// floats of scratch, scratch as for launch_argmax.
 cudaError_t launch_estimate(const void* B, int storage, const uint8_t* trav, const SessionDev* sd,
-                            float inv_uniform, int H, int W, int K, void* scratch, const long long* arg_idx,
-                            long long r2, int dk, double* partials, unsigned int nparts, EstimateOut* out,
-                            cudaStream_t st);
+                            float inv_uniform, int H, int W, int K, float* map, void* scratch, long long* arg_idx,
+                            float* arg_val, long long r2, int dk, double* partials, unsigned int nparts,
+                            EstimateOut* out, cudaStream_t st);
 // argmax_scratch_len(n) float + int pairs.
 size_t argmax_scratch_bytes(size_t n);
 cudaError_t launch_argmax(const void* B, int storage, const uint8_t* trav,

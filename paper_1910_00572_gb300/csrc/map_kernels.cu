@@ -207,15 +207,153 @@ __global__ void __launch_bounds__(NT) argmax_vec_kernel(const T* __restrict__ B,
     }
 }
 
-// loc_estimate: one pass over the belief around the argmax state a (written by the argmax
-// kernel on the same stream).  mass_near sums the states whose cell lies within the disk
-// dj^2 + di^2 <= r2 of a's cell and whose bin is within dk of a's (circular): FP32 Kahan per
-// thread, FP64 per CTA, the last CTA summing the CTA partials in a fixed order.  The second
-// hypothesis is the largest belief among the cells outside the disk, the lowest cell index on
-// ties (threads scan in increasing index order and combine with better()).
+// loc_estimate in two kernels.  The first reads the tensor once: the argmax state (as the argmax
+// pass finds it) and the stored belief map, max over bins, in map.  The second needs the tensor only
+// inside the estimate's disk and bins; the second hypothesis comes from the map.  What bounds them:
+// the one read.  (The argmax pass and a second pass over every state with its row, column and bin
+// took 18 + 39 us at 512 x 512 x 64 FP32; this form 23 + 10.)
+//
+// A CTA of 64 x 4 threads takes 64 groups of V consecutive cells, a quarter of the bins each.
+constexpr int MG = 64, MS = NT / MG;
+template <typename T, int V>
+__global__ void __launch_bounds__(NT) argmap_kernel(const T* __restrict__ B, const uint8_t* __restrict__ trav,
+                                                    const SessionDev* sd, float inv_uniform, size_t hw, int K,
+                                                    float* __restrict__ map, float* __restrict__ pv,
+                                                    long long* __restrict__ pi, unsigned int* counter,
+                                                    long long* out_idx, float* out_val) {
+    __shared__ float cv[MS][MG * V];
+    __shared__ int ck[MS][MG * V];
+    __shared__ float sv[NT / 32];
+    __shared__ long long si[NT / 32];
+    __shared__ int s_last;
+    const int gx = threadIdx.x % MG, part = threadIdx.x / MG;
+    const int k0 = (int)((long long)K * part / MS), k1 = (int)((long long)K * (part + 1) / MS);
+    const int reinit = sd->reinit;
+    const size_t ng = hw / V;
+    float bv = -FLT_MAX;
+    long long bi = LLONG_MAX;
+    for (size_t g0 = (size_t)blockIdx.x * MG; g0 < ng; g0 += (size_t)gridDim.x * MG) {
+        const size_t g = g0 + gx;
+        float v[V];
+        int kk[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            v[e] = -FLT_MAX;
+            kk[e] = k0;
+        }
+        if (g < ng) {
+            if (reinit) {                             // the belief reads as uniform over free cells
+#pragma unroll
+                for (int e = 0; e < V; ++e) v[e] = (float)trav[g * V + e] * inv_uniform;
+            } else {
+#pragma unroll 8
+                for (int k = k0; k < k1; ++k) {
+                    float x[V];
+                    if constexpr (V > 1) {
+                        union {
+                            uint4 u;
+                            T x[V];
+                        } raw;
+                        raw.u = __ldg(reinterpret_cast<const uint4*>(B + (size_t)k * hw) + g);
+#pragma unroll
+                        for (int e = 0; e < V; ++e) x[e] = Store<T>::ld(&raw.x[e]);
+                    } else {
+                        x[0] = Store<T>::ld(B + (size_t)k * hw + g);
+                    }
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        if (x[e] > v[e]) {            // the lowest bin among equal values
+                            v[e] = x[e];
+                            kk[e] = k;
+                        }
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            cv[part][gx * V + e] = v[e];
+            ck[part][gx * V + e] = kk[e];
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < MG * V; c += NT) {
+            const size_t cell = g0 * V + c;
+            if (cell < ng * V) {
+                float m = cv[0][c];
+                int k = ck[0][c];
+#pragma unroll
+                for (int q = 1; q < MS; ++q)
+                    if (cv[q][c] > m) {
+                        m = cv[q][c];
+                        k = ck[q][c];
+                    }
+                map[cell] = m;
+                const long long i = (long long)k * (long long)hw + (long long)cell;
+                if (better(m, i, bv, bi)) {
+                    bv = m;
+                    bi = i;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    auto reduce = [&]() {
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_down_sync(0xffffffffu, bv, o);
+            const long long oi = __shfl_down_sync(0xffffffffu, bi, o);
+            if (better(ov, oi, bv, bi)) {
+                bv = ov;
+                bi = oi;
+            }
+        }
+        if ((threadIdx.x & 31) == 0) {
+            sv[threadIdx.x >> 5] = bv;
+            si[threadIdx.x >> 5] = bi;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int w = 1; w < NT / 32; ++w)
+                if (better(sv[w], si[w], bv, bi)) {
+                    bv = sv[w];
+                    bi = si[w];
+                }
+        __syncthreads();
+    };
+    reduce();
+    if (threadIdx.x == 0) {
+        pv[blockIdx.x] = bv;
+        pi[blockIdx.x] = bi;
+        __threadfence();
+        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    bv = -FLT_MAX;
+    bi = LLONG_MAX;
+    for (unsigned int b = threadIdx.x; b < gridDim.x; b += NT) {
+        const float v = ((volatile float*)pv)[b];
+        const long long q = ((volatile long long*)pi)[b];
+        if (better(v, q, bv, bi)) {
+            bv = v;
+            bi = q;
+        }
+    }
+    reduce();
+    if (threadIdx.x == 0) {
+        *out_idx = bi;
+        *out_val = reinit ? bv : (float)((double)bv / sd->Z);
+        *counter = 0u;
+    }
+}
+
+// mass_near sums the states whose cell lies within the disk dj^2 + di^2 <= r2 of the argmax state's
+// cell and whose bin is within dk of its bin (circular): FP32 Kahan per thread, FP64 per CTA, the
+// last CTA summing the CTA partials in a fixed order.  The second hypothesis is the largest belief
+// among the cells outside the disk, the lowest cell index on ties.
 template <typename T>
 __global__ void __launch_bounds__(NT) estimate_kernel(const T* __restrict__ B, const uint8_t* __restrict__ trav,
-                                                      const SessionDev* sd, float inv_uniform, int H, int W, int K,
+                                                      const SessionDev* sd, float inv_uniform,
+                                                      const float* __restrict__ map, int H, int W, int K,
                                                       const long long* arg_idx, long long r2, int dk,
                                                       double* partials, float* pv, long long* pi,
                                                       unsigned int* counter, EstimateOut* out) {
@@ -230,167 +368,22 @@ __global__ void __launch_bounds__(NT) estimate_kernel(const T* __restrict__ B, c
     KahanF mass;
     float bv = -FLT_MAX;
     long long bi = LLONG_MAX;
-    // one thread per cell (consecutive across a warp), its K bins in turn
     for (size_t cell = (size_t)blockIdx.x * NT + threadIdx.x; cell < hw; cell += (size_t)gridDim.x * NT) {
         const int j = (int)(cell / (unsigned int)W), i = (int)(cell - (size_t)j * W);
         const long long dj = j - ja, di = i - ia;
-        const bool inside = dj * dj + di * di <= r2;
-        float m = 0.0f;                                   // the cell's belief-map value
-#pragma unroll 8
-        for (int k = 0; k < K; ++k) {
-            const float v = belief_at(B, trav, hw, (size_t)k * hw + cell, reinit, inv_uniform, scale);
-            if (inside) {
-                int d = k > ka ? k - ka : ka - k;
-                if (K - d < d) d = K - d;
-                if (d <= dk) mass.add(v);
-            } else {
-                m = fmaxf(m, v);
+        if (dj * dj + di * di <= r2) {
+            const int lo = 2 * (long long)dk + 1 < K ? ka - dk : 0, n = 2 * (long long)dk + 1 < K ? 2 * dk + 1 : K;
+#pragma unroll 4
+            for (int d = 0; d < n; ++d) {
+                int k = lo + d;
+                k = k < 0 ? k + K : k >= K ? k - K : k;
+                mass.add(belief_at(B, trav, hw, (size_t)k * hw + cell, reinit, inv_uniform, scale));
             }
-        }
-        if (!inside && better(m, (long long)cell, bv, bi)) {
-            bv = m;
-            bi = (long long)cell;
-        }
-    }
-    const double bm = block_sum<NT>(mass.value(), red);
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_down_sync(0xffffffffu, bv, o);
-        const long long oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (better(ov, oi, bv, bi)) {
-            bv = ov;
-            bi = oi;
-        }
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        sv[warp] = bv;
-        si[warp] = bi;
-    }
-    __syncthreads();
-    __shared__ int s_last;
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < NT / 32; ++w)
-            if (better(sv[w], si[w], bv, bi)) {
-                bv = sv[w];
-                bi = si[w];
-            }
-        partials[blockIdx.x] = bm;
-        pv[blockIdx.x] = bv;
-        pi[blockIdx.x] = bi;
-        __threadfence();
-        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    double ms = 0.0;
-    bv = -FLT_MAX;
-    bi = LLONG_MAX;
-    for (unsigned int b = threadIdx.x; b < gridDim.x; b += NT) {
-        ms += ((volatile double*)partials)[b];
-        const float v = ((volatile float*)pv)[b];
-        const long long q = ((volatile long long*)pi)[b];
-        if (better(v, q, bv, bi)) {
-            bv = v;
-            bi = q;
-        }
-    }
-    const double mt = block_sum<NT>(ms, red);
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_down_sync(0xffffffffu, bv, o);
-        const long long oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (better(ov, oi, bv, bi)) {
-            bv = ov;
-            bi = oi;
-        }
-    }
-    __syncthreads();
-    if (lane == 0) {
-        sv[warp] = bv;
-        si[warp] = bi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < NT / 32; ++w)
-            if (better(sv[w], si[w], bv, bi)) {
-                bv = sv[w];
-                bi = si[w];
-            }
-        out->mass_near = mt;
-        out->second_p = bv > 0.0f ? bv : 0.0f;
-        out->second_cell = bv > 0.0f ? bi : -1;
-        *counter = 0u;
-    }
-}
-
-// The same pass over the flat tensor in 16-byte groups of V consecutive states (hw a multiple
-// of V and W >= V, so a group stays in one plane): one division to place a thread's first
-// group, then the plane, cell, row and column advance by the grid stride.
-template <typename T, int V>
-__global__ void __launch_bounds__(NT) estimate_vec_kernel(const T* __restrict__ B, const uint8_t* __restrict__ trav,
-                                                          const SessionDev* sd, float inv_uniform, int H, int W,
-                                                          int K, const long long* arg_idx, long long r2, int dk,
-                                                          double* partials, float* pv, long long* pi,
-                                                          unsigned int* counter, EstimateOut* out) {
-    static_assert(V * sizeof(T) == 16, "one 16-byte load");
-    __shared__ double red[NT / 32];
-    __shared__ float sv[NT / 32];
-    __shared__ long long si[NT / 32];
-    const size_t hw = (size_t)H * W, ng = hw * K / V;
-    const long long a = *arg_idx;
-    const int ka = (int)(a / (long long)hw), ja = (int)((a % (long long)hw) / W), ia = (int)(a % W);
-    const int reinit = sd->reinit;
-    const float scale = sd->inv_Z;
-    KahanF mass;
-    float bv = -FLT_MAX;
-    long long bi = LLONG_MAX;
-    const size_t g0 = (size_t)blockIdx.x * NT + threadIdx.x, gs = (size_t)gridDim.x * NT;
-    if (g0 < ng) {
-        size_t q = g0 * V;
-        int k = (int)(q / hw);
-        size_t cell = q - (size_t)k * hw;
-        int j = (int)(cell / (unsigned int)W), i = (int)(cell - (size_t)j * W);
-        const size_t step = gs * V;                       // the grid stride in states
-        const int dkk = (int)(step / hw);
-        const size_t dcell = step - (size_t)dkk * hw;
-        const int dj = (int)(dcell / (unsigned int)W), di = (int)(dcell - (size_t)dj * W);
-        for (size_t g = g0; g < ng; g += gs) {
-            union {
-                uint4 u;
-                T x[V];
-            } raw;
-            if (!reinit) raw.u = __ldg(reinterpret_cast<const uint4*>(B) + g);
-            int je = j, ie = i;
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                if (e > 0 && ++ie == W) {
-                    ie = 0;
-                    ++je;
-                }
-                const size_t ce = cell + e;
-                const float v = reinit ? (float)trav[ce] * inv_uniform : Store<T>::ld(&raw.x[e]) * scale;
-                const long long ddj = je - ja, ddi = ie - ia;
-                if (ddj * ddj + ddi * ddi <= r2) {
-                    int d = k > ka ? k - ka : ka - k;
-                    if (K - d < d) d = K - d;
-                    if (d <= dk) mass.add(v);
-                } else if (better(v, (long long)ce, bv, bi)) {
-                    bv = v;
-                    bi = (long long)ce;
-                }
-            }
-            k += dkk;
-            cell += dcell;
-            j += dj;
-            i += di;
-            if (i >= W) {
-                i -= W;
-                ++j;
-            }
-            if (cell >= hw) {
-                cell -= hw;
-                j -= H;
-                ++k;
+        } else {
+            const float m = reinit ? map[cell] : map[cell] * scale;
+            if (better(m, (long long)cell, bv, bi)) {
+                bv = m;
+                bi = (long long)cell;
             }
         }
     }
@@ -620,28 +613,29 @@ cudaError_t launch_argmax(const void* B, int storage, const uint8_t* trav,
 }
 
 cudaError_t launch_estimate(const void* B, int storage, const uint8_t* trav, const SessionDev* sd,
-                            float inv_uniform, int H, int W, int K, void* scratch, const long long* arg_idx,
-                            long long r2, int dk, double* partials, unsigned int nparts, EstimateOut* out,
-                            cudaStream_t st) {
+                            float inv_uniform, int H, int W, int K, float* map, void* scratch, long long* arg_idx,
+                            float* arg_val, long long r2, int dk, double* partials, unsigned int nparts,
+                            EstimateOut* out, cudaStream_t st) {
     const size_t hw = (size_t)H * W;
     long long* pi = (long long*)scratch;
     float* pv = (float*)(pi + kArgmaxBlocks);
     unsigned int* counter = reinterpret_cast<unsigned int*>(pv + kArgmaxBlocks);
     const size_t vec = storage == LOC_F32 ? 4 : 8;
-    if (hw % vec == 0 && (size_t)W >= vec) {
-        unsigned int nb = grid_for(hw * K / vec);
-        if (nb > kArgmaxBlocks) nb = kArgmaxBlocks;
-        if (nb > nparts) nb = nparts;
-        LOC_DISPATCH(storage, (estimate_vec_kernel<T, 16 / sizeof(T)><<<nb, NT, 0, st>>>(
-                                  (const T*)B, trav, sd, inv_uniform, H, W, K, arg_idx, r2, dk, partials, pv, pi,
-                                  counter, out)));
-        return cudaGetLastError();
+    const size_t v = hw % vec == 0 ? vec : 1;
+    size_t na = (hw / v + MG - 1) / MG;
+    if (na > (size_t)kArgmaxBlocks) na = kArgmaxBlocks;
+    if (v > 1) {
+        LOC_DISPATCH(storage, (argmap_kernel<T, 16 / sizeof(T)><<<(unsigned int)na, NT, 0, st>>>(
+                                  (const T*)B, trav, sd, inv_uniform, hw, K, map, pv, pi, counter, arg_idx, arg_val)));
+    } else {
+        LOC_DISPATCH(storage, (argmap_kernel<T, 1><<<(unsigned int)na, NT, 0, st>>>(
+                                  (const T*)B, trav, sd, inv_uniform, hw, K, map, pv, pi, counter, arg_idx, arg_val)));
     }
-    unsigned int nb = grid_for(hw);
-    if (nb > kArgmaxBlocks) nb = kArgmaxBlocks;
+    unsigned int nb = grid_for(hw);                   // few CTAs: the last one gathers their results
+    if (nb > 304) nb = 304;
     if (nb > nparts) nb = nparts;
-    LOC_DISPATCH(storage, (estimate_kernel<T><<<nb, NT, 0, st>>>((const T*)B, trav, sd, inv_uniform, H, W, K, arg_idx,
-                                                                 r2, dk, partials, pv, pi, counter, out)));
+    LOC_DISPATCH(storage, (estimate_kernel<T><<<nb, NT, 0, st>>>((const T*)B, trav, sd, inv_uniform, map, H, W, K,
+                                                                 arg_idx, r2, dk, partials, pv, pi, counter, out)));
     return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ struct loc_session {
     long long* argmax_idx = nullptr;
     float* argmax_val = nullptr;
     unsigned char* pinned = nullptr;   // 64 bytes of pinned host memory for small readbacks
+    float* map_buf = nullptr;          // [H][W] of readback scratch (allocated on first use)
     loc::EstimateOut* est = nullptr;   // loc_estimate's device results (allocated on first use)
     // LIDAR sample update scratch (allocated on first use)
     bool lidar_ready = false;
