@@ -181,6 +181,7 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
             it.partials = S.partials;
             it.log_out_mult = S.log_out_mult;
         },
+        []() {}, [](stream::Item&, stream::Source&) {},
         [&](const stream::Item& it, int slot) {
             if (dry) return;
             stream::retire_tile<false>(sm, it, slot, it.partials, nullptr, nullptr, &it.sd->counter,

@@ -15,9 +15,11 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const uint32_t sbase = su32(smem_raw);
     stream::Smem<T>& sm = *reinterpret_cast<stream::Smem<T>*>(smem_raw + (((sbase + 127u) & ~127u) - sbase));
-    const int reinit = a.sd->reinit;
-    // restart: the input is M / (K n_free); read M and fold 1 / (K n_free) into the scale
-    const float in_scale = (reinit ? a.inv_uniform : a.sd->inv_Z) * a.out_mult;
+    // The next step's CTAs may take the SMs that this one's leave: their barriers, plans and masks
+    // (all from the map and the launch's arguments) are then ready when the grid ends.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    int reinit = 0;
+    float in_scale = 0.0f;
     int tile = blockIdx.x;
     run_roles<T, AM, RAG>(
         sm,
@@ -25,7 +27,6 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
             if (tile >= ntiles) return;
             it.out = a.B_out;
             it.in = a.B_in;
-            it.reinit = reinit;
             it.trav = a.trav;
             it.corr = a.corr;
             it.K = a.K;
@@ -33,7 +34,6 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
             it.W = a.W;
             it.ty0 = (tile / ntx) * stream::TH;
             it.tx0 = (tile % ntx) * TW;
-            it.in_scale = in_scale;
             it.g0 = a.g0;
             it.g1 = a.g1;
             it.g2 = a.g2;
@@ -43,8 +43,18 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
             it.ntiles = ntiles;
             src.tmap = &a.tmap;
             src.sh = a.sh;
-            src.reinit = reinit;
             tile += gridDim.x;
+        },
+        [&]() {
+            // what earlier work on the stream wrote is read (and overwritten) from here on
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            reinit = a.sd->reinit;
+            // restart: the input is M / (K n_free); read M and fold 1 / (K n_free) into the scale
+            in_scale = (reinit ? a.inv_uniform : a.sd->inv_Z) * a.out_mult;
+        },
+        [&](Item& it, Source& src) {
+            it.in_scale = in_scale;
+            it.reinit = src.reinit = reinit;
         },
         [&](const Item& it, int slot) {
             retire_tile<AM>(sm, it, slot, a.partials, a.am_pv, a.am_pi, &a.sd->counter, [&](double Z, const ArgBest& b) {
@@ -76,8 +86,17 @@ cudaError_t launch(const FastArgs& a, cudaStream_t st) {
     }
     const int ntx = (a.W + TW - 1) / TW, ntiles = ntx * ((a.H + stream::TH - 1) / stream::TH);
     const int grid = ntiles < sms[slot] ? ntiles : sms[slot];
-    step_stream_kernel<T, AM, RAG><<<grid, stream::NT, sb, st>>>(a, ntx, ntiles);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(stream::NT);
+    cfg.dynamicSmemBytes = sb;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, step_stream_kernel<T, AM, RAG>, a, ntx, ntiles);
 }
 
 }  // namespace

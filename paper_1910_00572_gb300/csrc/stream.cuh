@@ -869,10 +869,12 @@ __device__ __forceinline__ void retire_tile(const SM& sm, const Item& it, int sl
     }
 }
 
-// The roles of the CTA's warps; next and done as for manage().  The first tile is set up by all
-// of them: the manager's planes travel while the others read the map.
-template <typename T, bool AM, bool RAG, typename Next, typename Done>
-__device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Done done) {
+// The roles of the CTA's warps; next and done as for manage().  next() gives a tile's geometry and
+// input(item, src) what earlier work on the stream wrote (scale, restart flag); for the first tile
+// begin() runs between them, the barriers, the plan and the map mask being set up by then: the
+// manager's planes travel while the other warps read the map.
+template <typename T, bool AM, bool RAG, typename Next, typename Begin, typename Input, typename Done>
+__device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Begin begin, Input input, Done done) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Item it{};
     Source src{};
@@ -886,16 +888,26 @@ __device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Done done) {
     }
     __syncthreads();
     if (warp != NO) {
-        const Item t = sm.item[0];
+        const Item& t = sm.item[0];
         if (t.K) fill_mask<NT - 32, RAG>(sm, 0, t, warp < NO ? threadIdx.x : threadIdx.x - 32);
         asm volatile("bar.sync 1, %0;" ::"n"(NT - 32) : "memory");
-    } else if (lane == 0) {
-        arrive(&sm.it_full[0]);
+    } else {
+        begin();
+        input(it, src);
+        if (lane == 0) {
+            sm.item[0].in_scale = it.in_scale;
+            sm.item[0].reinit = it.reinit;
+            arrive(&sm.it_full[0]);
+        }
+        __syncwarp();
     }
     if (warp < NO + 1) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsOut));
         if (warp < NO) output<T, AM, RAG>(sm, threadIdx.x);
-        else manage<T, RAG>(sm, it, src, next, done);
+        else manage<T, RAG>(sm, it, src, [&](Item& t, Source& s) {
+            next(t, s);
+            input(t, s);
+        }, done);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsBlur));
         blur<T, RAG>(sm, warp - (NO + 1));
