@@ -81,7 +81,8 @@ __global__ void __launch_bounds__(NT) belief_map_vec_kernel(const T* __restrict_
 #pragma unroll
             for (int e = 0; e < V; ++e) v[e] = (float)trav[g * V + e] * inv_uniform;
         } else {
-            for (int k = 0; k < K; ++k) {
+#pragma unroll 8
+            for (int k = 0; k < K; ++k) {                      // eight planes' loads in flight
                 union {
                     uint4 u;
                     T x[V];
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(NT) belief_map_vec_kernel(const T* __restrict_
 // the whole map is a wavefront of W + 94 + (blocks - 1) x (94 + hand-off) steps.  One CTA of 16
 // warps (four rows of blocks one after the other, 16 warps on four schedulers, a fence per
 // hand-off) took 1.73 ms at 2048 x 2048; a warp per block on a scheduler of its own, with
-// hand-offs that need no fence, takes 0.42 (66 cycles a step, ten thousand cycles from a block's
+// hand-offs that need no fence, takes 0.40 (60-odd cycles a step, ten thousand cycles from a block's
 // start to the next one's).  The cluster keeps the warps that wait on one another resident together.
 //
 // Hand-off: a block's last lane writes its errors into the next block's inbox as it goes: shared
@@ -177,12 +178,14 @@ __global__ void __launch_bounds__(kFsWarps * 64) fs_kernel(const float* __restri
     auto await = [&](auto ready) {
         if (ready()) return;
         const unsigned long long g0 = gtime();
-        for (unsigned int it = 0; !ready();)
+        for (unsigned int it = 0; !ready();) {
+            if (loader) __nanosleep(200);                      // two chunks ahead: leave the pipes to the steps
             if (__any_sync(0xffffffffu, ++it > (1u << 24) || gtime() - g0 > wait_ns)) {
                 if (lane == 0) atomicOr(status, LOC_DEV_ERR_TIMEOUT);
                 failed = true;                                 // the blocks below run into their limits too
                 return;
             }
+        }
     };
     int round = 0;
     for (int rb = blockIdx.x * kFsWarps + warp; rb < nrb && !failed; rb += gridDim.x * kFsWarps, ++round) {
