@@ -203,9 +203,9 @@ def profiled_traffic(wl, args):
     if wl["name"] != "office512" or wl["storage"] != "f32" or args.tile not in (0, 16) or args.kernel not in (0, 2):
         return None
     try:
-        text = open(os.path.join(ROOT, "profiles", "step_ws_office512.md")).read()
+        text = open(os.path.join(ROOT, "profiles", "step_stream_office512.md")).read()
         csrc = os.path.join(ROOT, "paper_1910_00572_gb300", "csrc")
-        src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("tiled_common.cuh", "step_tiled.cu"))
+        src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("tiled_common.cuh", "stream.cuh", "step_stream.cu"))
     except OSError:
         return None
     sha = re.search(r"source_sha256:\s*([0-9a-f]+)", text)
@@ -227,7 +227,7 @@ def served_traffic(alg_bytes_per_launch):
     try:
         text = open(os.path.join(ROOT, "profiles", "batch_kernel_batch64_bf16.md")).read()
         csrc = os.path.join(ROOT, "paper_1910_00572_gb300", "csrc")
-        src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("tiled_common.cuh", "batch.cu"))
+        src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("tiled_common.cuh", "stream.cuh", "batch.cu"))
     except OSError:
         return None
     sha = re.search(r"source_sha256:\s*([0-9a-f]+)", text)
@@ -409,8 +409,8 @@ def measure_single(args, wl, occ, walk, ws, rank, local, cpu_budget_s=15.0):
         "gpu_launches": args.steps,
         "clocks": clk.summary(),
         "last_Z": stats["last_Z"],
-        "estimate_readback": {"ms": float(np.median(est_ms)), "kernels": "argmax + estimate (two passes)",
-                              "achieved_gbs": 2 * n_cells * elem / (float(np.median(est_ms)) / 1e3) / 1e9,
+        "estimate_readback": {"ms": float(np.median(est_ms)), "kernels": "argmax and belief map (one read), estimate",
+                              "achieved_gbs": n_cells * elem / (float(np.median(est_ms)) / 1e3) / 1e9,
                               "note": "device time of loc_estimate(0.5 m, 2 bins) incl. its pinned readback"},
     }
     return line

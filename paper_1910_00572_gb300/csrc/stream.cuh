@@ -15,15 +15,18 @@
 //
 // RAG: rows whose pitch is no multiple of 16 bytes.  TMA cannot address them, so each blur warp
 // brings its own plane (load_rows); the stores are single values, and the operations follow the
-// generic kernel's order, whose place it takes (613 x 797 x 48 FP32: 634 -> 84 us).
+// generic kernel's order, whose place it takes (613 x 797 x 48 FP32: 634 -> 79 us).
 //
 // Why this split.  The tile body it replaces ran S, X and P as passes of all warps through
 // shared memory with two CTA barriers a plane: 42 to 53 thread instructions a cell and issue
-// 41 to 52 % busy.  Here a plane costs about 20 (FP32) to 28 (BF16) instructions a cell, eight
+// 41 to 52 % busy.  Here a cell costs 35 (FP32) to 39 (BF16), eight
 // planes are in the works at once, and the latency of one plane's chain no longer counts.
 // Every value is computed with the operations and the order of the passes in tiled_common.cuh,
 // and a thread of the output warps sums the same cells, so tensors and normalisers are those
-// of the 128-thread synchronous configuration bit for bit.
+// of the 128-thread synchronous configuration bit for bit.  Before and after, us a step: 64 x 64 x
+// 16 FP32 27.3 -> 16.7, 500 x 500 x 128 111 -> 64, 512 x 512 x 64 63.5 -> 39.7, 1816 x 1816 x 36 FP16
+// 310 -> 253, 2048 x 2048 x 72 BF16 725 -> 550 (2.2 TB/s) and FP32 793 -> 543 (4.5 TB/s).  What bounds
+// it now: the output warps' instruction issue and latency, two of them on a scheduler.
 #pragma once
 #include <type_traits>
 
@@ -39,7 +42,6 @@ constexpr int XR = TH + 2 * R;         // 32 rows of S and X: one per lane
 constexpr int RAW_H = XR + 1;          // raw rows
 constexpr int NB = 8;                  // blur warps = raw stages = X planes in flight
 constexpr int NO = 7;                  // output warps
-constexpr int NTP = NO * 32;           // output threads
 constexpr int NT = 32 * (1 + NB + NO); // 512
 constexpr int SQ = 17;                 // quads of S columns (68 = 64 + 4)
 constexpr int XPAD = 4;                // columns in front of an X row's 64
