@@ -20,7 +20,7 @@ __all__ = [
     "loc_params_default", "loc_set_allocator", "loc_create", "loc_step", "loc_lidar_update",
     "loc_lidar_update_cells", "loc_belief", "loc_marginal", "loc_argmax", "loc_set_belief",
     "loc_stats", "loc_sync", "loc_destroy", "loc_last_error", "torch_stream",
-    "use_torch_allocator", "loc_propagate_noalloc", "loc_debug_fs_stall", "loc_samples", "loc_dither", "loc_ray_ranges",
+    "use_torch_allocator", "loc_propagate_noalloc", "loc_debug_fs_stall", "loc_debug_step_stall", "loc_samples", "loc_dither", "loc_ray_ranges",
     "loc_range_table", "loc_range_table_read", "loc_lidar_update_dense", "loc_estimate", "loc_map_difficulty",
     "loc_estimate_t",
     "LOC_BATCH_CONFIGS", "Batch", "loc_batch_create", "loc_batch_step", "loc_batch_sync",
@@ -125,6 +125,7 @@ _SIGS = {
     "loc_destroy": (ctypes.c_int, [_P]),
     "loc_last_error": (ctypes.c_char_p, [_P]),
     "loc_debug_fs_stall": (ctypes.c_int, [ctypes.c_int, ctypes.c_double]),
+    "loc_debug_step_stall": (ctypes.c_int, [ctypes.c_int]),
     "loc_propagate_noalloc": (ctypes.c_int, [ctypes.POINTER(loc_params), _P, _P, _P, _P,
                                              ctypes.c_double, ctypes.c_double]),
     "loc_samples": (ctypes.c_int, [_P, _P, ctypes.c_size_t, ctypes.POINTER(ctypes.c_int)]),
@@ -399,6 +400,11 @@ def loc_last_error(h: Handle | None = None) -> str:
 def loc_debug_fs_stall(stall: bool, wait_limit_s: float = 0.2) -> None:
     """Test hook: make the dithering's bounded block hand-offs wait on a flag nothing sets."""
     _check(None, lib().loc_debug_fs_stall(1 if stall else 0, float(wait_limit_s)))
+
+
+def loc_debug_step_stall(tile: int) -> None:
+    """Test hook: the streaming propagation withholds each CTA's tile-th tile (0: off)."""
+    _check(None, lib().loc_debug_step_stall(int(tile)))
 
 
 def loc_propagate_noalloc(params: loc_params, occ_dev: int, b_in_dev: int, b_out_dev: int,

@@ -127,6 +127,8 @@ batch_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restrict__ t
     }
 }
 
+__device__ int g_stall = 0;                // see set_batch_stall
+
 // The same queue for the streaming tiles (stream.cuh): the manager warp takes the items, so the
 // next item's planes are in flight while the CTA finishes the previous one.
 template <typename T>
@@ -139,7 +141,7 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
     const int lane = threadIdx.x & 31;
     const int total = list->total, n_active = list->n_active;
     stream::run_roles<T, false, false>(
-        sm,
+        sm, g_stall,
         [&](stream::Item& it, stream::Source& src) {
             int q = 0;
             if (lane == 0) q = atomicAdd(&ctl->head, 1);
@@ -190,8 +192,7 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
     if (threadIdx.x == 0 && sm.fail) {
         // flag the launch and the sessions of the tiles in work; their Z is not updated
         atomicOr(&ctl->status, LOC_DEV_ERR_TIMEOUT);
-        for (int k = 0; k < 2; ++k)
-            if (sm.item[k].K > 0) atomicOr(&sm.item[k].sd->status, LOC_DEV_ERR_TIMEOUT);
+        stream::flag_failed(sm);
     }
 }
 
@@ -268,6 +269,8 @@ cudaError_t launch_cfg(int cfg, int grid, const BatchStatic* ss, const void* tic
 size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 }  // namespace
+
+cudaError_t set_batch_stall(int tile) { return cudaMemcpyToSymbol(g_stall, &tile, sizeof(tile)); }
 
 int batch_num_cfgs() { return 3; }
 

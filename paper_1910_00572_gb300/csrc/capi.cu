@@ -631,6 +631,14 @@ LOC_API loc_status loc_debug_fs_stall(int stall, double wait_limit_s) {
     return LOC_OK;
 }
 
+LOC_API loc_status loc_debug_step_stall(int tile) {
+    if (tile < 0) return fail(nullptr, LOC_ERR_INVALID_ARG, "tile must be >= 0");
+    cudaError_t e = set_step_stall(tile);
+    if (e == cudaSuccess) e = set_batch_stall(tile);
+    if (e != cudaSuccess) return fail(nullptr, LOC_ERR_CUDA, std::string("loc_debug_step_stall: ") + cudaGetErrorString(e));
+    return LOC_OK;
+}
+
 LOC_API loc_status loc_lidar_update(loc_handle h, const float* ranges, int n_beams, double angle_min,
                                     double angle_inc, double r_max, int beam_stride, double sigma_r) {
     loc_status st = check_live(h);

@@ -63,6 +63,11 @@ cudaError_t launch_step_stream(const void* args, int storage, bool argmax, cudaS
 bool step_ragged_eligible(int K, int r_xy, int r_th);
 cudaError_t launch_step_ragged(const StepArgs& a, int storage, cudaStream_t st);
 int stream_tile_rows();
+// Test hook of the streaming kernels' bounded waits, in every later launch of the single-session
+// (set_step_stall) and of the batched form (set_batch_stall): a CTA's tile-th tile is never handed
+// to its warps, whose waits run out; 0: off.
+cudaError_t set_step_stall(int tile);
+cudaError_t set_batch_stall(int tile);
 int stream_box_w(int storage);
 cudaError_t launch_step_tiled(const StepArgs& a, const void* tmap, int storage, int cfg, cudaStream_t st);
 

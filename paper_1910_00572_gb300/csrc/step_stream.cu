@@ -9,6 +9,8 @@ namespace {
 
 using namespace stream;
 
+__device__ int g_stall = 0;                // see set_step_stall
+
 template <typename T, bool AM, bool RAG>
 __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid_constant__ FastArgs a, int ntx,
                                                                     int ntiles) {
@@ -22,7 +24,7 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
     float in_scale = 0.0f;
     int tile = blockIdx.x;
     run_roles<T, AM, RAG>(
-        sm,
+        sm, g_stall,
         [&](Item& it, Source& src) {
             if (tile >= ntiles) return;
             it.out = a.B_out;
@@ -122,6 +124,8 @@ cudaError_t launch_step_ragged(const StepArgs& g, int storage, cudaStream_t st) 
         default: return cudaErrorInvalidValue;
     }
 }
+
+cudaError_t set_step_stall(int tile) { return cudaMemcpyToSymbol(g_stall, &tile, sizeof(tile)); }
 
 bool step_ragged_eligible(int K, int r_xy, int r_th) { return r_xy == R && r_th == RT && K >= 8 && K <= LOC_MAX_K; }
 

@@ -90,6 +90,7 @@ struct Smem {
     float am_v[2][NO];                 // ... and argmax candidates
     long long am_i[2][NO];
     volatile int fail;                 // a bounded wait gave up: every warp leaves its loop
+    SessionDev* held;                  // session of the tile that the manager took but has not published
 };
 
 __device__ __forceinline__ void arrive(unsigned long long* b) {
@@ -381,6 +382,9 @@ __device__ __forceinline__ void init_barriers(Smem<T>& sm) {
         bar_init(&sm.it_empty[s], NB + NO);
     }
     sm.fail = 0;
+    // a CTA that gives up reads both slots (flag_failed), the second one perhaps before it held a tile
+    sm.item[0].K = sm.item[1].K = 0;
+    sm.held = nullptr;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -439,9 +443,10 @@ __device__ __forceinline__ void fill_plan(SM& sm, int slot, const Item& t, const
 
 // Manager warp, with the first item published in slot 0 (its plan too).  next(item, src) (all
 // lanes, the same answer) gives the next tile or K = 0; done(item, slot) (all lanes) takes a
-// finished tile's sums out of its slot.
+// finished tile's sums out of its slot.  stall: the CTA's stall-th tile is never handed over (a
+// test of the bounded waits; 0: none).
 template <typename T, bool RAG, typename Next, typename Done>
-__device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next next, Done done) {
+__device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, int stall, Next next, Done done) {
     constexpr uint32_t kBoxBytes = RAW_H * box_w<T>() * sizeof(T);
     constexpr int AL = align_elems<T>();
     const int lane = threadIdx.x & 31;
@@ -485,10 +490,17 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
             fill_plan<RAG>(sm, slot, t, from, lane);
             fill_mask<32, RAG>(sm, slot, t, lane);
         }
-        if (lane == 0) sm.item[slot] = t;
+        if (lane == 0) {
+            sm.item[slot] = t;
+            sm.held = nullptr;
+        }
         __syncwarp();
-        if (lane == 0) arrive(&sm.it_full[slot]);
+        if (lane == 0 && stall != (int)i + 1) arrive(&sm.it_full[slot]);
         return true;
+    };
+    auto take = [&](Item& t, Source& from) {
+        next(t, from);
+        if (lane == 0 && t.K) sm.held = t.sd;
     };
     bool ok = true;
     unsigned int i = 0;
@@ -496,12 +508,12 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
         Item nit{};
         Source nsrc{};
         if constexpr (RAG) {           // the blur warps bring the planes
-            next(nit, nsrc);
+            take(nit, nsrc);
             ok = publish(i + 1, nit, nsrc);
         } else for (int p = 0; ok && p < it.K; ++p) {
             ok = issue(p);
             if (ok && p == (it.K > NB ? NB : it.K - 1)) {   // early in the tile: the next one
-                next(nit, nsrc);
+                take(nit, nsrc);
                 ok = publish(i + 1, nit, nsrc);
             }
         }
@@ -871,12 +883,21 @@ __device__ __forceinline__ void retire_tile(const SM& sm, const Item& it, int sl
     }
 }
 
-// The roles of the CTA's warps; next and done as for manage().  next() gives a tile's geometry and
+// After run_roles, by one thread of a CTA that gave up: flags the sessions of every tile that it took
+// and whose sums it did not record, which are those in the slots and the one in the manager's hands.
+template <typename SM>
+__device__ __forceinline__ void flag_failed(const SM& sm) {
+    for (int k = 0; k < 2; ++k)
+        if (sm.item[k].K > 0) atomicOr(&sm.item[k].sd->status, LOC_DEV_ERR_TIMEOUT);
+    if (sm.held) atomicOr(&sm.held->status, LOC_DEV_ERR_TIMEOUT);
+}
+
+// The roles of the CTA's warps; next, done and stall as for manage().  next() gives a tile's geometry and
 // input(item, src) what earlier work on the stream wrote (scale, restart flag); for the first tile
 // begin() runs between them, the barriers, the plan and the map mask being set up by then: the
 // manager's planes travel while the other warps read the map.
 template <typename T, bool AM, bool RAG, typename Next, typename Begin, typename Input, typename Done>
-__device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Begin begin, Input input, Done done) {
+__device__ __forceinline__ void run_roles(Smem<T>& sm, int stall, Next next, Begin begin, Input input, Done done) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Item it{};
     Source src{};
@@ -899,14 +920,14 @@ __device__ __forceinline__ void run_roles(Smem<T>& sm, Next next, Begin begin, I
         if (lane == 0) {
             sm.item[0].in_scale = it.in_scale;
             sm.item[0].reinit = it.reinit;
-            arrive(&sm.it_full[0]);
+            if (stall != 1) arrive(&sm.it_full[0]);
         }
         __syncwarp();
     }
     if (warp < NO + 1) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsOut));
         if (warp < NO) output<T, AM, RAG>(sm, threadIdx.x);
-        else manage<T, RAG>(sm, it, src, [&](Item& t, Source& s) {
+        else manage<T, RAG>(sm, it, src, stall, [&](Item& t, Source& s) {
             next(t, s);
             input(t, s);
         }, done);
