@@ -33,6 +33,7 @@
 
 #include "dda.cuh"
 #include "kernels.h"
+#include "per_device.h"
 #include "tiled_common.cuh"
 
 namespace loc {
@@ -380,15 +381,17 @@ template <typename T, int NB, bool FULL>
 cudaError_t score_nb(const uint8_t* table, const uint8_t* trav, const void* B, size_t hw, int K, int A, const int* m,
                      const float* zs, int nu, float scale, float* logL, unsigned int* maxL, cudaStream_t st) {
     const size_t smem = dense_score_smem(A, K, nu);
-    static size_t attr[64] = {};                   // per device: the largest size set so far
-    int dev = 0;
+    // one size for every launch: with the launch's own, a thread with a small table could lower the limit
+    // between another's setting it and its launch
+    static PerDevice ready;
+    int dev = 0, set = 0;
     cudaGetDevice(&dev);
-    if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || smem > attr[dev])) {
-        const cudaError_t e = cudaFuncSetAttribute(dense_score_kernel<T, NB, FULL>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr[dev] = smem;
-    }
+    const cudaError_t e = ready.get(dev, &set, [](int* n) {
+        *n = 1;
+        return cudaFuncSetAttribute(dense_score_kernel<T, NB, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)dense_score_smem(LOC_MAX_TABLE_DIRS, 1, LOC_MAX_DENSE_BEAMS));
+    });
+    if (e != cudaSuccess) return e;
     const unsigned int nb = (unsigned int)((hw + DC - 1) / DC);
     dense_score_kernel<T, NB, FULL><<<nb, SNT, smem, st>>>(table, trav, static_cast<const T*>(B), hw, K, A, A / K, m, zs, nu,
                                                      scale, logL, maxL);

@@ -13,6 +13,7 @@
 
 #include "dda.cuh"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace loc {
 namespace {
@@ -689,26 +690,24 @@ cudaError_t launch_belief_map(const void* B, int storage, const uint8_t* trav, S
 cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_t* selbits, int* rowcnt, int* rowoff,
                           int* count, float* bnd, int* status, int cap, int32_t* samples, cudaStream_t st) {
     const int nrb = (H + 31) / 32;
-    static int max_ctas[64] = {};                              // per device: the largest cluster it can hold
-    int dev = 0;
+    static PerDevice largest;                                  // cluster that the device can hold
+    int dev = 0, max_ctas = 0;
     cudaGetDevice(&dev);
-    const int slot = dev >= 0 && dev < 64 ? dev : 0;
-    cudaError_t e = cudaSuccess;
-    if (slot != dev || !max_ctas[slot]) {
+    cudaError_t e = largest.get(dev, &max_ctas, [](int* n) {
         const int most = (int)(kFsRingBytes + kFsInboxBytes);
+        cudaError_t e = cudaSuccess;
         for (auto* f : {fs_kernel<true>, fs_kernel<false>}) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         }
-        if (e != cudaSuccess) return e;
-        int n = kFsMaxCtas, fit = 0;
-        for (; n > 1; n /= 2) {
+        int fit = 0;
+        for (*n = kFsMaxCtas; e == cudaSuccess && *n > 1; *n /= 2) {
             cudaLaunchConfig_t q{};
             cudaLaunchAttribute qa{};
             qa.id = cudaLaunchAttributeClusterDimension;
-            qa.val.clusterDim.x = n;
+            qa.val.clusterDim.x = *n;
             qa.val.clusterDim.y = qa.val.clusterDim.z = 1;
-            q.gridDim = dim3(n);
+            q.gridDim = dim3(*n);
             q.blockDim = dim3(kFsWarps * 64);
             q.dynamicSmemBytes = most;
             q.attrs = &qa;
@@ -716,10 +715,11 @@ cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_
             if (cudaOccupancyMaxActiveClusters(&fit, fs_kernel<true>, &q) == cudaSuccess && fit > 0) break;
             cudaGetLastError();
         }
-        max_ctas[slot] = n;
-    }
+        return e;
+    });
+    if (e != cudaSuccess) return e;
     int ctas = 1;                                              // a power of two, one warp per block
-    while (ctas < max_ctas[slot] && ctas * kFsWarps < nrb) ctas *= 2;
+    while (ctas < max_ctas && ctas * kFsWarps < nrb) ctas *= 2;
     // the inboxes in shared memory where the rows fit
     const int nbox = ctas * kFsWarps < nrb ? 2 : 1;
     const size_t boxes = sizeof(float) * kFsWarps * nbox * (size_t)((W + 31) / 32 * 32 + 64);

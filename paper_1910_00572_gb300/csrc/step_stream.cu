@@ -2,6 +2,7 @@
 // dealt to the persistent CTAs in turn.
 #include <type_traits>
 
+#include "per_device.h"
 #include "stream.cuh"
 
 namespace loc {
@@ -78,20 +79,17 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
 
 template <typename T, bool AM, bool RAG = false>
 cudaError_t launch(const FastArgs& a, cudaStream_t st) {
-    static bool attr_set[64] = {};
-    static int sms[64] = {};
-    int dev = 0;
+    static PerDevice sms;
+    int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
-    const int slot = dev >= 0 && dev < 64 ? dev : 0;
     const size_t sb = sizeof(stream::Smem<T>) + 128;
-    if (slot != dev || !attr_set[slot]) {
-        cudaError_t e = prepare<T>(step_stream_kernel<T, AM, RAG>);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms[slot], cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        attr_set[slot] = true;
-    }
+    const cudaError_t e = sms.get(dev, &n_sm, [dev](int* n) {
+        const cudaError_t p = prepare<T>(step_stream_kernel<T, AM, RAG>);
+        return p != cudaSuccess ? p : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+    });
+    if (e != cudaSuccess) return e;
     const int ntx = (a.W + TW - 1) / TW, ntiles = ntx * ((a.H + stream::TH - 1) / stream::TH);
-    const int grid = ntiles < sms[slot] ? ntiles : sms[slot];
+    const int grid = ntiles < n_sm ? ntiles : n_sm;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(stream::NT);
