@@ -346,9 +346,9 @@ loc_status loc_batch_destroy(loc_batch b);
 /* Description of the batch's last failure ("" if none; b may be NULL). */
 const char* loc_batch_last_error(loc_batch b);
 
-/* Device bytes a session created with p holds once it has run a LIDAR update (the belief
- * tensors, map, correction, reduction and sampling scratch, each allocation rounded up to
- * 512 bytes).  Used for admission against a memory budget.  No device work. */
+/* Device bytes a session created with p holds once it has run a LIDAR update and been read out
+ * (the belief tensors, map, correction, reduction, sampling and readout scratch, each allocation
+ * rounded up to 512 bytes).  Used for admission against a memory budget.  No device work. */
 loc_status loc_session_bytes(const loc_params* p, size_t* bytes);
 
 /* ---- Serving loop: many robot sessions stepped as their messages arrive (continuous batching).

@@ -175,11 +175,10 @@ LOC_API loc_status loc_session_bytes(const loc_params* p, size_t* bytes) {
     size_t cap = 2 * (size_t)p->n_samples + 4 * (H + W) + 1024;
     if (cap > hw) cap = hw;
     const size_t nrb = (H + 31) / 32;
-    // (the selections take an eighth of the hw bytes counted for them: room for the tables that a
-    // scan of more beams grows)
-    b += r(hw * 4) + r(hw) + 2 * r(H * 4) + r((nrb + 1) * W * 4) + r((nrb + 2) * 4) + r(cap * 4) +
-         r(cap * K * 4) + r(64) + r(reweight_scalars_bytes()) + r(K * 1080 * 8) + r(1080 * 4) + r(K * 1080 * 4) +
-         r(H * ((W + 31) / 32) * 4);
+    // (the map m also serves the readouts; the selections and the map's bits are a word per 32 cells)
+    b += r(hw * 4) + 2 * r(H * ((W + 31) / 32) * 4) + 2 * r(H * 4) + r((nrb + 1) * W * 4) + r(cap * 4) +
+         r(cap * K * 4) + r(64) + r(reweight_scalars_bytes()) + r(K * 1080 * 8) + r(1080 * 4) + r(K * 1080 * 4);
+    b += r(sizeof(EstimateOut));
     *bytes = b;
     return LOC_OK;
 }
@@ -415,6 +414,14 @@ LOC_API loc_status loc_step(loc_handle h, double u, double v, double w) {
 
 namespace {
 
+// The session's [H][W] floats of scratch, allocated on first use: the belief map that a scan selects
+// its samples from, and what loc_marginal and loc_estimate read back.  Nothing in it outlives a call,
+// and all its uses are on the session's stream.
+bool map_scratch(loc_session* h) {
+    if (!h->m) h->m = (float*)dev_alloc(h, h->hw * sizeof(float));
+    return h->m != nullptr;
+}
+
 loc_status lidar_setup(loc_session* h) {
     if (h->lidar_ready) return LOC_OK;
     const int H = h->p.H, W = h->p.W, K = h->p.K;
@@ -423,7 +430,6 @@ loc_status lidar_setup(loc_session* h) {
     if (cap > hw) cap = hw;
     h->cap = (int)cap;
     const int nrb = (H + 31) / 32;
-    h->m = (float*)dev_alloc(h, sizeof(float) * hw);
     h->travbits = (uint32_t*)dev_alloc(h, sizeof(uint32_t) * (size_t)H * ((W + 31) / 32));
     h->sel = (uint32_t*)dev_alloc(h, sizeof(uint32_t) * (size_t)H * ((W + 31) / 32));
     h->rowcnt = (int*)dev_alloc(h, sizeof(int) * H);
@@ -433,7 +439,7 @@ loc_status lidar_setup(loc_session* h) {
     h->logL = (float*)dev_alloc(h, sizeof(float) * (size_t)cap * K);
     h->dscal = (int*)dev_alloc(h, 64);
     h->rs = dev_alloc(h, reweight_scalars_bytes());
-    if (!h->m || !h->sel || !h->rowcnt || !h->rowoff || !h->bnd || !h->samples || !h->logL ||
+    if (!map_scratch(h) || !h->sel || !h->rowcnt || !h->rowoff || !h->bnd || !h->samples || !h->logL ||
         !h->dscal || !h->rs || !h->travbits)
         return fail(h, LOC_ERR_OOM, "LIDAR scratch allocation failed");
     cudaError_t e = cudaMemsetAsync(h->dscal, 0, 64, h->stream);
@@ -968,13 +974,6 @@ LOC_API loc_status loc_map_difficulty(loc_handle h, const int32_t* probes, int n
     return sync_and_check(h);
 }
 
-// The session's H * W floats of readback scratch, allocated on first use (all its uses are on the
-// session's stream).
-static bool map_buffer(loc_session* h) {
-    if (!h->map_buf) h->map_buf = (float*)dev_alloc(h, h->hw * sizeof(float));
-    return h->map_buf != nullptr;
-}
-
 LOC_API loc_status loc_belief(loc_handle h, float* out, size_t n) {
     loc_status st = check_live(h);
     if (st != LOC_OK) return st;
@@ -996,10 +995,10 @@ LOC_API loc_status loc_marginal(loc_handle h, float* out, size_t n, int mode) {
     if (st != LOC_OK) return st;
     if (!out || n != h->hw) return fail(h, LOC_ERR_INVALID_ARG, "out null or n != H*W");
     if (mode != LOC_MAP_SUM && mode != LOC_MAP_MAX) return fail(h, LOC_ERR_INVALID_ARG, "mode");
-    if (!map_buffer(h)) return fail(h, LOC_ERR_OOM, "readback buffer");
+    if (!map_scratch(h)) return fail(h, LOC_ERR_OOM, "readback buffer");
     cudaError_t e = launch_read_marginal(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform,
-                                         h->p.H, h->p.W, h->p.K, mode, h->map_buf, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, h->map_buf, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
+                                         h->p.H, h->p.W, h->p.K, mode, h->m, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, h->m, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_marginal");
     return sync_and_check(h);
 }
@@ -1053,13 +1052,13 @@ LOC_API loc_status loc_estimate(loc_handle h, double radius_m, int dk, loc_estim
         h->est = (EstimateOut*)dev_alloc(h, sizeof(EstimateOut));
         if (!h->est) return fail(h, LOC_ERR_OOM, "estimate buffer");
     }
-    if (!map_buffer(h)) return fail(h, LOC_ERR_OOM, "estimate buffer");
+    if (!map_scratch(h)) return fail(h, LOC_ERR_OOM, "estimate buffer");
     const double c = h->p.cell_m;
     // cells whose centres lie within radius_m; the 1e-9 keeps a whole number of cells inclusive
     const double r2d = std::floor(radius_m * radius_m / (c * c) + 1e-9);
     const long long r2 = r2d > 4.0e18 ? (long long)4e18 : (long long)r2d;
     cudaError_t e = launch_estimate(h->B[h->cur], h->p.storage, h->trav, h->sd, h->inv_uniform, h->p.H, h->p.W, h->p.K,
-                                    h->map_buf, h->argmax_scratch, h->argmax_idx, h->argmax_val, r2, dk, h->partials,
+                                    h->m, h->argmax_scratch, h->argmax_idx, h->argmax_val, r2, dk, h->partials,
                                     h->nparts, h->est, h->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->pinned, h->argmax_idx, sizeof(long long) + sizeof(float), cudaMemcpyDeviceToHost,

@@ -38,12 +38,11 @@ struct loc_session {
     long long* argmax_idx = nullptr;
     float* argmax_val = nullptr;
     unsigned char* pinned = nullptr;   // 64 bytes of pinned host memory for small readbacks
-    float* map_buf = nullptr;          // [H][W] of readback scratch (allocated on first use)
     loc::EstimateOut* est = nullptr;   // loc_estimate's device results (allocated on first use)
     // LIDAR sample update scratch (allocated on first use)
     bool lidar_ready = false;
     int cap = 0;                   // capacity of the sample list
-    float* m = nullptr;            // belief map [H][W]
+    float* m = nullptr;            // belief map [H][W] (also the readouts' scratch: map_scratch)
     uint32_t* travbits = nullptr;  // the map as bits [H][ceil(W / 32)] (the ray casts' window)
     uint32_t* sel = nullptr;       // selections as bits [H][ceil(W / 32)]
     int* rowcnt = nullptr;         // per-row selections [H]
