@@ -120,7 +120,8 @@ enum { LOC_KERNEL_AUTO = 0, LOC_KERNEL_GENERIC = 1, LOC_KERNEL_TILED = 2 };
 void loc_params_default(loc_params* p);
 
 /* Optional device allocator for every later loc_create.  alloc(bytes, stream, ctx) returns
- * a device pointer or NULL; release(ptr, stream, ctx) frees it.  Pass NULLs to go back to
+ * a device pointer or NULL; release(ptr, stream, ctx) frees it.  A pointer that is no multiple of
+ * 16 is released and 15 bytes more are asked for.  Pass NULLs to go back to
  * cudaMalloc/cudaFree.  Not thread-safe with concurrent loc_create/loc_destroy. */
 typedef void* (*loc_alloc_fn)(size_t bytes, void* stream, void* ctx);
 typedef void (*loc_free_fn)(void* ptr, void* stream, void* ctx);

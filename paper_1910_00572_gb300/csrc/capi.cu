@@ -43,16 +43,35 @@ loc_status cuda_fail(loc_session* s, cudaError_t e, const char* what) {
     return fail(s, LOC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Device memory of the session, aligned to kDevAlign.  A registered allocator may hand out any
+// address: one that is not aligned goes back, and the same request with room to align follows.
+constexpr size_t kDevAlign = 16;           // the widest load of the kernels; what TMA asks of a base
+
 void* dev_alloc(loc_session* s, size_t bytes) {
-    void* p = nullptr;
+    void* base = nullptr;
     if (g_alloc) {
-        p = g_alloc(bytes, (void*)s->stream, g_alloc_ctx);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        base = g_alloc(bytes, (void*)s->stream, g_alloc_ctx);
+        if ((uintptr_t)base % kDevAlign) {
+            g_free(base, (void*)s->stream, g_alloc_ctx);
+            base = g_alloc(bytes + kDevAlign - 1, (void*)s->stream, g_alloc_ctx);
+        }
+    } else if (cudaMalloc(&base, bytes) != cudaSuccess) {
         cudaGetLastError();
-        p = nullptr;
+        base = nullptr;
     }
-    if (p) s->owned.push_back(p);
+    if (!base) return nullptr;
+    void* p = (void*)(((uintptr_t)base + kDevAlign - 1) / kDevAlign * kDevAlign);
+    s->owned.push_back(DevBlock{p, base});
     return p;
+}
+
+void dev_release(loc_session* s, void* p) {
+    auto it = std::find_if(s->owned.begin(), s->owned.end(), [p](const DevBlock& b) { return b.p == p; });
+    if (it == s->owned.end()) return;
+    void* base = it->base;
+    s->owned.erase(it);
+    if (g_free) g_free(base, (void*)s->stream, g_alloc_ctx);
+    else cudaFree(base);
 }
 
 void release_all(loc_session* s) {
@@ -67,11 +86,7 @@ void release_all(loc_session* s) {
         s->scan_pin[k] = nullptr;
         s->scan_pin_ev[k] = nullptr;
     }
-    for (void* p : s->owned) {
-        if (g_free) g_free(p, (void*)s->stream, g_alloc_ctx);
-        else cudaFree(p);
-    }
-    s->owned.clear();
+    while (!s->owned.empty()) dev_release(s, s->owned.front().p);
 }
 
 void taps(double sigma, int r, float* out) {
@@ -448,14 +463,6 @@ loc_status lidar_setup(loc_session* h) {
     if (e != cudaSuccess) return cuda_fail(h, e, "LIDAR scratch init");
     h->lidar_ready = true;
     return LOC_OK;
-}
-
-void dev_release(loc_session* h, void* p) {
-    auto it = std::find(h->owned.begin(), h->owned.end(), p);
-    if (it == h->owned.end()) return;
-    h->owned.erase(it);
-    if (g_free) g_free(p, (void*)h->stream, g_alloc_ctx);
-    else cudaFree(p);
 }
 
 // Grow a device buffer to at least n elements of `elem` bytes (the old one is released).
@@ -984,8 +991,7 @@ LOC_API loc_status loc_belief(loc_handle h, float* out, size_t n) {
                                        h->p.H, h->p.W, h->p.K, tmp, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->owned.pop_back();
-    if (g_free) g_free(tmp, (void*)h->stream, g_alloc_ctx); else cudaFree(tmp);
+    dev_release(h, tmp);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_belief");
     return sync_and_check(h);
 }
@@ -1112,8 +1118,7 @@ LOC_API loc_status loc_set_belief(loc_handle h, const float* b, size_t n) {
     if (e == cudaSuccess)
         e = launch_set_belief(tmp, h->B[h->cur], h->p.storage, n, h->sd, h->partials, h->nparts, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->owned.pop_back();
-    if (g_free) g_free(tmp, (void*)h->stream, g_alloc_ctx); else cudaFree(tmp);
+    dev_release(h, tmp);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_set_belief");
     return sync_and_check(h);
 }

@@ -8,6 +8,13 @@
 #include "kernels.h"
 #include "loc.h"
 
+namespace loc {
+struct DevBlock {                      // a device buffer p and the pointer that the allocator gave for it
+    void* p;
+    void* base;
+};
+}  // namespace loc
+
 struct loc_session {
     loc_params p{};
     int r_xy = 0, r_th = 0;
@@ -84,7 +91,7 @@ struct loc_session {
     long long n_prop = 0;
     bool failed = false;
     std::string err;
-    std::vector<void*> owned;
+    std::vector<loc::DevBlock> owned;
 };
 
 
@@ -93,6 +100,7 @@ namespace loc {
 loc_status fail(loc_session* s, loc_status code, const std::string& msg);
 loc_status cuda_fail(loc_session* s, cudaError_t e, const char* what);
 void* dev_alloc(loc_session* s, size_t bytes);
+void dev_release(loc_session* s, void* p);
 void release_all(loc_session* s);
 loc_status check_live(loc_session* h);
 // Kernel radius for sigma (given >= 0 overrides), as loc_create derives it.
