@@ -747,16 +747,15 @@ LOC_API loc_status loc_dither(loc_handle h, const float* m, float fs, uint8_t* s
     if (e == cudaSuccess)
         e = launch_dither(h->m, reinterpret_cast<float*>(h->dscal + 2), h->p.H, h->p.W, h->sel, h->rowcnt, h->rowoff,
                           h->dscal + 3, h->bnd, &h->sd->status, 0, nullptr, h->stream);
-    const int H = h->p.H, W = h->p.W, nch = (W + 31) / 32;
-    std::vector<uint32_t> bits((size_t)H * nch);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(bits.data(), h->sel, sizeof(uint32_t) * bits.size(), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(count, h->dscal + 3, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    // the map has been read: its buffer takes the selections as bytes
+    uint8_t* bytes = reinterpret_cast<uint8_t*>(h->m);
+    if (e == cudaSuccess) e = launch_unpack_bits(h->sel, h->p.H, h->p.W, bytes, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sel, bytes, h->hw, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->pinned, h->dscal + 3, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "loc_dither");
-    for (int j = 0; j < H; ++j)
-        for (int i = 0; i < W; ++i) sel[(size_t)j * W + i] = (bits[(size_t)j * nch + (i >> 5)] >> (i & 31)) & 1u;
-    return sync_and_check(h);
+    st = sync_and_check(h);                    // one wait for the count and the status
+    std::memcpy(count, h->pinned, sizeof(int));
+    return st;
 }
 
 LOC_API loc_status loc_ray_ranges(loc_handle h, const int32_t* cells, int n_cells, const float* dirs, int n_dirs,

@@ -171,6 +171,8 @@ cudaError_t launch_belief_map(const void* B, int storage, const uint8_t* trav, S
 // raster-ordered list of at most cap selected linear indices.  bnd holds ceil(H / 32) * W floats.
 cudaError_t launch_dither(const float* m, const float* fs, int H, int W, uint32_t* selbits, int* rowcnt, int* rowoff,
                           int* count, float* bnd, int* status, int cap, int32_t* samples, cudaStream_t st);
+// Those bits as one byte a cell, [H][W].
+cudaError_t launch_unpack_bits(const uint32_t* bits, int H, int W, uint8_t* out, cudaStream_t st);
 cudaError_t launch_ray_ranges(const uint8_t* trav, int H, int W, const int32_t* cells, int n_cells, const float* dirs,
                               int n_dirs, float rmax_cells, float cell_m, float* out, cudaStream_t st);
 size_t reweight_scalars_bytes();

@@ -400,6 +400,18 @@ __global__ void __launch_bounds__(1024) row_scan_kernel(const int* __restrict__ 
     if (threadIdx.x == 1023) *count = part[1023];
 }
 
+// Selections as one byte a cell, for loc_dither's caller (with a loop over the bits on the host the call took
+// 3.6 ms at 2048 x 2048, 2.0 like this).
+__global__ void __launch_bounds__(NT) unpack_bits_kernel(const uint32_t* __restrict__ bits, size_t hw, int W,
+                                                         uint8_t* __restrict__ out) {
+    const int nch = (W + 31) / 32;
+    for (size_t q = (size_t)blockIdx.x * NT + threadIdx.x; q < hw; q += (size_t)gridDim.x * NT) {
+        const size_t j = q / W;
+        const int i = (int)(q - j * W);
+        out[q] = (bits[j * nch + (i >> 5)] >> (i & 31)) & 1u;
+    }
+}
+
 // Linear indices of the selected cells in raster order (one warp per row, a word of 32 selections
 // a lane), at most cap.
 __global__ void __launch_bounds__(NT) compact_kernel(const uint32_t* __restrict__ selbits, const int* __restrict__ rowoff,
@@ -751,6 +763,11 @@ cudaError_t set_fs_wait(double seconds, int stall) {
     cudaError_t e = cudaMemcpyToSymbol(g_fs_wait_ns, &ns, sizeof(ns));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_fs_stall, &stall, sizeof(stall));
     return e;
+}
+
+cudaError_t launch_unpack_bits(const uint32_t* bits, int H, int W, uint8_t* out, cudaStream_t st) {
+    unpack_bits_kernel<<<grid_for((size_t)H * W, 4096), NT, 0, st>>>(bits, (size_t)H * W, W, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ray_ranges(const uint8_t* trav, int H, int W, const int32_t* cells, int n_cells, const float* dirs,
