@@ -210,74 +210,89 @@ __global__ void __launch_bounds__(NT) argmax_vec_kernel(const T* __restrict__ B,
 // loc_estimate in two kernels.  The first reads the tensor once: the argmax state (as the argmax
 // pass finds it) and the stored belief map, max over bins, in map.  The second needs the tensor only
 // inside the estimate's disk and bins; the second hypothesis comes from the map.  What bounds them:
-// the one read.  (The argmax pass and a second pass over every state with its row, column and bin
-// took 18 + 39 us at 512 x 512 x 64 FP32; this form 23 + 10.)
+// the one read.  The argmax pass and a second pass over every state with its row, column and bin
+// took 17 + 39 us at 512 x 512 x 64 FP32; this form 20 + 9 with a small disk, 20 + 20 with one over the
+// whole map.
 //
-// A CTA of 64 x 4 threads takes 64 groups of V consecutive cells, a quarter of the bins each.
+// A CTA of 64 x 4 threads takes 64 E cells, a quarter of the bins each: a thread E consecutive cells
+// where rows of E are aligned to 16 bytes (VEC), else E cells 64 apart, one load each.  Eight bins' loads
+// are in flight, the last bin again past the quarter's end (a loop over what is left took its loads one
+// by one).  613 x 797 x 48 FP32 67 -> 32 us, 1001 x 1003 x 24 BF16 95 -> 30 (one cell a thread before),
+// 1024 x 1024 x 64 BF16 61 -> 37.
 constexpr int MG = 64, MS = NT / MG;
-template <typename T, int V>
+template <typename T, int E, bool VEC>
 __global__ void __launch_bounds__(NT) argmap_kernel(const T* __restrict__ B, const uint8_t* __restrict__ trav,
                                                     const SessionDev* sd, float inv_uniform, size_t hw, int K,
                                                     float* __restrict__ map, float* __restrict__ pv,
                                                     long long* __restrict__ pi, unsigned int* counter,
                                                     long long* out_idx, float* out_val) {
-    __shared__ float cv[MS][MG * V];
-    __shared__ int ck[MS][MG * V];
+    static_assert(!VEC || E * sizeof(T) == 16, "one 16-byte load");
+    __shared__ float cv[MS][MG * E];
+    __shared__ int ck[MS][MG * E];
     __shared__ float sv[NT / 32];
     __shared__ long long si[NT / 32];
     __shared__ int s_last;
     const int gx = threadIdx.x % MG, part = threadIdx.x / MG;
     const int k0 = (int)((long long)K * part / MS), k1 = (int)((long long)K * (part + 1) / MS);
     const int reinit = sd->reinit;
-    const size_t ng = hw / V;
     float bv = -FLT_MAX;
     long long bi = LLONG_MAX;
-    for (size_t g0 = (size_t)blockIdx.x * MG; g0 < ng; g0 += (size_t)gridDim.x * MG) {
-        const size_t g = g0 + gx;
-        float v[V];
-        int kk[V];
+    for (size_t c0 = (size_t)blockIdx.x * MG * E; c0 < hw; c0 += (size_t)gridDim.x * MG * E) {
+        auto local = [&](int e) { return VEC ? gx * E + e : gx + MG * e; };
+        float v[E];
+        int kk[E];
+        bool in[E];
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
+        for (int e = 0; e < E; ++e) {
             v[e] = -FLT_MAX;
             kk[e] = k0;
+            in[e] = c0 + local(e) < hw;               // VEC: hw is a multiple of E, all or none
         }
-        if (g < ng) {
-            if (reinit) {                             // the belief reads as uniform over free cells
+        if (reinit) {                                 // the belief reads as uniform over free cells
 #pragma unroll
-                for (int e = 0; e < V; ++e) v[e] = (float)trav[g * V + e] * inv_uniform;
-            } else {
-#pragma unroll 8
-                for (int k = k0; k < k1; ++k) {
-                    float x[V];
-                    if constexpr (V > 1) {
+            for (int e = 0; e < E; ++e)
+                if (in[e]) v[e] = (float)trav[c0 + local(e)] * inv_uniform;
+        } else if (in[0]) {
+            const T* p[VEC ? 1 : E];
+#pragma unroll
+            for (int e = 0; e < (VEC ? 1 : E); ++e) p[e] = B + c0 + local(in[e] ? e : 0);
+            for (int kb = k0; kb < k1; kb += 8) {
+                float x[8][E];
+#pragma unroll
+                for (int d = 0; d < 8; ++d) {
+                    const size_t at = (size_t)min(kb + d, k1 - 1) * hw;
+                    if constexpr (VEC) {
                         union {
                             uint4 u;
-                            T x[V];
+                            T x[E];
                         } raw;
-                        raw.u = __ldg(reinterpret_cast<const uint4*>(B + (size_t)k * hw) + g);
+                        raw.u = __ldg(reinterpret_cast<const uint4*>(p[0] + at));
 #pragma unroll
-                        for (int e = 0; e < V; ++e) x[e] = Store<T>::ld(&raw.x[e]);
+                        for (int e = 0; e < E; ++e) x[d][e] = Store<T>::ld(&raw.x[e]);
                     } else {
-                        x[0] = Store<T>::ld(B + (size_t)k * hw + g);
-                    }
 #pragma unroll
-                    for (int e = 0; e < V; ++e)
-                        if (x[e] > v[e]) {            // the lowest bin among equal values
-                            v[e] = x[e];
-                            kk[e] = k;
-                        }
+                        for (int e = 0; e < E; ++e) x[d][e] = Store<T>::ld(p[e] + at);
+                    }
                 }
+#pragma unroll
+                for (int d = 0; d < 8; ++d)
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (x[d][e] > v[e]) {         // the lowest bin among equal values
+                            v[e] = x[d][e];
+                            kk[e] = kb + d;
+                        }
             }
         }
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-            cv[part][gx * V + e] = v[e];
-            ck[part][gx * V + e] = kk[e];
+        for (int e = 0; e < E; ++e) {
+            cv[part][local(e)] = v[e];
+            ck[part][local(e)] = kk[e];
         }
         __syncthreads();
-        for (int c = threadIdx.x; c < MG * V; c += NT) {
-            const size_t cell = g0 * V + c;
-            if (cell < ng * V) {
+        for (int c = threadIdx.x; c < MG * E; c += NT) {
+            const size_t cell = c0 + c;
+            if (cell < hw) {
                 float m = cv[0][c];
                 int k = ck[0][c];
 #pragma unroll
@@ -349,8 +364,9 @@ __global__ void __launch_bounds__(NT) argmap_kernel(const T* __restrict__ B, con
 // mass_near sums the states whose cell lies within the disk dj^2 + di^2 <= r2 of the argmax state's
 // cell and whose bin is within dk of its bin (circular): FP32 Kahan per thread, FP64 per CTA, the
 // last CTA summing the CTA partials in a fixed order.  The second hypothesis is the largest belief
-// among the cells outside the disk, the lowest cell index on ties.
-template <typename T>
+// among the cells outside the disk, the lowest cell index on ties.  A thread takes V neighbouring cells,
+// eight bins' loads in flight.
+template <typename T, int V>
 __global__ void __launch_bounds__(NT) estimate_kernel(const T* __restrict__ B, const uint8_t* __restrict__ trav,
                                                       const SessionDev* sd, float inv_uniform,
                                                       const float* __restrict__ map, int H, int W, int K,
@@ -368,23 +384,59 @@ __global__ void __launch_bounds__(NT) estimate_kernel(const T* __restrict__ B, c
     KahanF mass;
     float bv = -FLT_MAX;
     long long bi = LLONG_MAX;
-    for (size_t cell = (size_t)blockIdx.x * NT + threadIdx.x; cell < hw; cell += (size_t)gridDim.x * NT) {
-        const int j = (int)(cell / (unsigned int)W), i = (int)(cell - (size_t)j * W);
-        const long long dj = j - ja, di = i - ia;
-        if (dj * dj + di * di <= r2) {
-            const int lo = 2 * (long long)dk + 1 < K ? ka - dk : 0, n = 2 * (long long)dk + 1 < K ? 2 * dk + 1 : K;
-#pragma unroll 4
-            for (int d = 0; d < n; ++d) {
-                int k = lo + d;
+    const bool some = 2 * (long long)dk + 1 < K;      // not all bins: dk either side of ka
+    const int lo = some ? ka - dk : 0, n = some ? 2 * dk + 1 : K;
+    for (size_t cell = V * ((size_t)blockIdx.x * NT + threadIdx.x); cell < hw; cell += V * (size_t)gridDim.x * NT) {
+        int j = (int)(cell / (unsigned int)W), i = (int)(cell - (size_t)j * W);
+        bool in[V], any = false;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const long long dj = j - ja, di = i - ia;
+            in[e] = dj * dj + di * di <= r2;
+            any |= in[e];
+            if (!in[e]) {
+                const float m = reinit ? map[cell + e] : map[cell + e] * scale;
+                if (better(m, (long long)(cell + e), bv, bi)) {
+                    bv = m;
+                    bi = (long long)(cell + e);
+                }
+            }
+            if (V > 1 && ++i == W) {
+                i = 0;
+                ++j;
+            }
+        }
+        if (!any) continue;
+        for (int d0 = 0; d0 < n; d0 += 8) {
+            float v[8][V];
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                int k = lo + min(d0 + d, n - 1);          // past the last bin it again, not added
                 k = k < 0 ? k + K : k >= K ? k - K : k;
-                mass.add(belief_at(B, trav, hw, (size_t)k * hw + cell, reinit, inv_uniform, scale));
+                const size_t q = (size_t)k * hw + cell;
+                if constexpr (V > 1) {
+                    union {
+                        uint4 u;
+                        T x[V];
+                    } raw;
+                    raw.u = __ldg(reinterpret_cast<const uint4*>(B + q));
+#pragma unroll
+                    for (int e = 0; e < V; ++e) v[d][e] = Store<T>::ld(&raw.x[e]) * scale;
+                } else {
+                    v[d][0] = Store<T>::ld(B + q) * scale;
+                }
             }
-        } else {
-            const float m = reinit ? map[cell] : map[cell] * scale;
-            if (better(m, (long long)cell, bv, bi)) {
-                bv = m;
-                bi = (long long)cell;
+            if (reinit) {                                 // the belief reads as uniform over free cells
+#pragma unroll
+                for (int d = 0; d < 8; ++d)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) v[d][e] = (float)trav[cell + e] * inv_uniform;
             }
+#pragma unroll
+            for (int d = 0; d < 8; ++d)
+#pragma unroll
+                for (int e = 0; e < V; ++e)
+                    if (d0 + d < n && in[e]) mass.add(v[d][e]);
         }
     }
     const double bm = block_sum<NT>(mass.value(), red);
@@ -622,20 +674,33 @@ cudaError_t launch_estimate(const void* B, int storage, const uint8_t* trav, con
     unsigned int* counter = reinterpret_cast<unsigned int*>(pv + kArgmaxBlocks);
     const size_t vec = storage == LOC_F32 ? 4 : 8;
     const size_t v = hw % vec == 0 ? vec : 1;
-    size_t na = (hw / v + MG - 1) / MG;
+    constexpr int kScalar = 4;                        // cells a thread without 16-byte loads
+    const size_t tile = MG * (v > 1 ? v : (size_t)kScalar);
+    size_t na = (hw + tile - 1) / tile;
     if (na > (size_t)kArgmaxBlocks) na = kArgmaxBlocks;
     if (v > 1) {
-        LOC_DISPATCH(storage, (argmap_kernel<T, 16 / sizeof(T)><<<(unsigned int)na, NT, 0, st>>>(
+        LOC_DISPATCH(storage, (argmap_kernel<T, 16 / sizeof(T), true><<<(unsigned int)na, NT, 0, st>>>(
                                   (const T*)B, trav, sd, inv_uniform, hw, K, map, pv, pi, counter, arg_idx, arg_val)));
     } else {
-        LOC_DISPATCH(storage, (argmap_kernel<T, 1><<<(unsigned int)na, NT, 0, st>>>(
+        LOC_DISPATCH(storage, (argmap_kernel<T, kScalar, false><<<(unsigned int)na, NT, 0, st>>>(
                                   (const T*)B, trav, sd, inv_uniform, hw, K, map, pv, pi, counter, arg_idx, arg_val)));
     }
-    unsigned int nb = grid_for(hw);                   // few CTAs: the last one gathers their results
-    if (nb > 304) nb = 304;
+    // The second pass takes 16-byte groups where they give every SM work (1024 x 1024 x 64 BF16, disk over
+    // the whole map: 44 us against 152 with a cell a thread; 512 x 512 x 24 13 against 24), and a cell a
+    // thread on smaller maps (256 x 256 x 36 BF16, 8192 groups: 14 against 16).
+    const size_t w = v > 1 && hw / v >= 32768 ? v : 1;
+    unsigned int nb = grid_for(hw / w);
+    if (nb > (unsigned int)kArgmaxBlocks) nb = kArgmaxBlocks;
     if (nb > nparts) nb = nparts;
-    LOC_DISPATCH(storage, (estimate_kernel<T><<<nb, NT, 0, st>>>((const T*)B, trav, sd, inv_uniform, map, H, W, K,
-                                                                 arg_idx, r2, dk, partials, pv, pi, counter, out)));
+    if (w > 1) {
+        LOC_DISPATCH(storage, (estimate_kernel<T, 16 / sizeof(T)><<<nb, NT, 0, st>>>(
+                                  (const T*)B, trav, sd, inv_uniform, map, H, W, K, arg_idx, r2, dk, partials, pv, pi,
+                                  counter, out)));
+    } else {
+        LOC_DISPATCH(storage, (estimate_kernel<T, 1><<<nb, NT, 0, st>>>(
+                                  (const T*)B, trav, sd, inv_uniform, map, H, W, K, arg_idx, r2, dk, partials, pv, pi,
+                                  counter, out)));
+    }
     return cudaGetLastError();
 }
 
