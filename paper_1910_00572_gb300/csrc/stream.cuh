@@ -722,10 +722,16 @@ __device__ __forceinline__ void output(Smem<T>& sm, int t) {
                 else st[rr] = put2<T>(out[rr], fmul2(cs[rr], v), res[rr], on[rr]);
                 out[rr] += plane;
             }
-            f2 part = st[0];
+            if constexpr (RAG) {                         // two values a compensated addition, as the generic kernel
+                static_assert(MR % 2 == 0, "pairs of rows");
 #pragma unroll
-            for (int rr = 1; rr < MR; ++rr) part = fadd2(part, st[rr]);
-            acc.add(part);
+                for (int rr = 0; rr < MR; rr += 2) acc.add(fadd2(st[rr], st[rr + 1]));
+            } else {
+                f2 part = st[0];
+#pragma unroll
+                for (int rr = 1; rr < MR; ++rr) part = fadd2(part, st[rr]);
+                acc.add(part);
+            }
             if constexpr (AM) {
                 float m = -FLT_MAX;
 #pragma unroll
