@@ -470,10 +470,10 @@ const char* loc_server_last_error(loc_server s);
 loc_status loc_debug_fs_stall(int stall, double wait_limit_s);
 
 /* The same for the streaming propagation (loc_step's tile configurations 3, 16 and 17, rows that
- * TMA does not apply to, and batches of configuration 3): with tile = n >= 1 every thread block
- * withholds the n-th tile that it takes from the warps that wait for it.  Their waits run out after
- * 0.2 s; the sessions of the block's unfinished tiles fail with LOC_ERR_TIMEOUT.  tile = 0 restores
- * the default.  Errors: INVALID_ARG (tile < 0), CUDA. */
+ * TMA does not apply to, and batches of configuration 3): with tile 1 or 2 every thread block
+ * withholds the first or second tile that it takes from the warps that wait for it.  Their waits run
+ * out after 0.2 s; the sessions of the block's unfinished tiles fail with LOC_ERR_TIMEOUT.  tile = 0
+ * restores the default.  Errors: INVALID_ARG (another tile), CUDA. */
 loc_status loc_debug_step_stall(int tile);
 
 /* Wait for all enqueued work of the handle; returns the first device-side error if any. */

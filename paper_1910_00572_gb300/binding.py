@@ -403,7 +403,7 @@ def loc_debug_fs_stall(stall: bool, wait_limit_s: float = 0.2) -> None:
 
 
 def loc_debug_step_stall(tile: int) -> None:
-    """Test hook: the streaming propagation withholds each CTA's tile-th tile (0: off)."""
+    """Test hook: the streaming propagation withholds each CTA's first or second tile (1, 2; 0: off)."""
     _check(None, lib().loc_debug_step_stall(int(tile)))
 
 

@@ -127,7 +127,7 @@ batch_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restrict__ t
     }
 }
 
-__device__ int g_stall = 0;                // see set_batch_stall
+__constant__ int g_stall = 0;              // see set_batch_stall
 
 // The same queue for the streaming tiles (stream.cuh): the manager warp takes the items, so the
 // next item's planes are in flight while the CTA finishes the previous one.
@@ -140,7 +140,8 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
     stream::Smem<T>& sm = *reinterpret_cast<stream::Smem<T>*>(smem_raw + (((base + 127u) & ~127u) - base));
     const int lane = threadIdx.x & 31;
     const int total = list->total, n_active = list->n_active;
-    stream::run_roles<T, false, false>(
+    if (threadIdx.x == 0) stream::none_taken(sm);
+    stream::run_roles<T, false, false, true>(
         sm, g_stall,
         [&](stream::Item& it, stream::Source& src) {
             int q = 0;

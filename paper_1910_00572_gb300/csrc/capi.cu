@@ -645,7 +645,7 @@ LOC_API loc_status loc_debug_fs_stall(int stall, double wait_limit_s) {
 }
 
 LOC_API loc_status loc_debug_step_stall(int tile) {
-    if (tile < 0) return fail(nullptr, LOC_ERR_INVALID_ARG, "tile must be >= 0");
+    if (tile < 0 || tile > 2) return fail(nullptr, LOC_ERR_INVALID_ARG, "tile must be 0, 1 or 2");
     cudaError_t e = set_step_stall(tile);
     if (e == cudaSuccess) e = set_batch_stall(tile);
     if (e != cudaSuccess) return fail(nullptr, LOC_ERR_CUDA, std::string("loc_debug_step_stall: ") + cudaGetErrorString(e));

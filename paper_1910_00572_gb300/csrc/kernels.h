@@ -64,8 +64,8 @@ bool step_ragged_eligible(int K, int r_xy, int r_th);
 cudaError_t launch_step_ragged(const StepArgs& a, int storage, cudaStream_t st);
 int stream_tile_rows();
 // Test hook of the streaming kernels' bounded waits, in every later launch of the single-session
-// (set_step_stall) and of the batched form (set_batch_stall): a CTA's tile-th tile is never handed
-// to its warps, whose waits run out; 0: off.
+// (set_step_stall) and of the batched form (set_batch_stall): a CTA's first (1) or second (2) tile is
+// never handed to its warps, whose waits run out; 0: off.
 cudaError_t set_step_stall(int tile);
 cudaError_t set_batch_stall(int tile);
 int stream_box_w(int storage);

@@ -10,7 +10,7 @@ namespace {
 
 using namespace stream;
 
-__device__ int g_stall = 0;                // see set_step_stall
+__constant__ int g_stall = 0;              // see set_step_stall
 
 template <typename T, bool AM, bool RAG>
 __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid_constant__ FastArgs a, int ntx,
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(stream::NT, 1) step_stream_kernel(const __grid
     int reinit = 0;
     float in_scale = 0.0f;
     int tile = blockIdx.x;
-    run_roles<T, AM, RAG>(
+    run_roles<T, AM, RAG, false>(
         sm, g_stall,
         [&](Item& it, Source& src) {
             if (tile >= ntiles) return;

@@ -90,7 +90,7 @@ struct Smem {
     float am_v[2][NO];                 // ... and argmax candidates
     long long am_i[2][NO];
     volatile int fail;                 // a bounded wait gave up: every warp leaves its loop
-    SessionDev* held;                  // session of the tile that the manager took but has not published
+    SessionDev* held;                  // QUEUE: session of the tile that the manager took but has not published
 };
 
 __device__ __forceinline__ void arrive(unsigned long long* b) {
@@ -369,8 +369,10 @@ struct Source {
     int reinit;                        // read the input as M (uniform restart) instead of TMA
 };
 
+// stall: the CTA's first (1) or second (2) tile is never handed over, since its barrier waits for one
+// arrival more than comes (a test of the bounded waits); 0: none.
 template <typename T>
-__device__ __forceinline__ void init_barriers(Smem<T>& sm) {
+__device__ __forceinline__ void init_barriers(Smem<T>& sm, int stall) {
     for (int s = 0; s < NB; ++s) {
         bar_init(&sm.raw_full[s], 1);
         bar_init(&sm.raw_empty[s], 1);
@@ -378,13 +380,10 @@ __device__ __forceinline__ void init_barriers(Smem<T>& sm) {
         bar_init(&sm.x_empty[s], NO);
     }
     for (int s = 0; s < 2; ++s) {
-        bar_init(&sm.it_full[s], 1);
+        bar_init(&sm.it_full[s], stall == s + 1 ? 2 : 1);
         bar_init(&sm.it_empty[s], NB + NO);
     }
     sm.fail = 0;
-    // a CTA that gives up reads both slots (flag_failed), the second one perhaps before it held a tile
-    sm.item[0].K = sm.item[1].K = 0;
-    sm.held = nullptr;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -443,10 +442,10 @@ __device__ __forceinline__ void fill_plan(SM& sm, int slot, const Item& t, const
 
 // Manager warp, with the first item published in slot 0 (its plan too).  next(item, src) (all
 // lanes, the same answer) gives the next tile or K = 0; done(item, slot) (all lanes) takes a
-// finished tile's sums out of its slot.  stall: the CTA's stall-th tile is never handed over (a
-// test of the bounded waits; 0: none).
-template <typename T, bool RAG, typename Next, typename Done>
-__device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, int stall, Next next, Done done) {
+// finished tile's sums out of its slot.  QUEUE: the tiles are of several sessions, so the one in
+// hand is kept for flag_failed.
+template <typename T, bool RAG, bool QUEUE, typename Next, typename Done>
+__device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next next, Done done) {
     constexpr uint32_t kBoxBytes = RAW_H * box_w<T>() * sizeof(T);
     constexpr int AL = align_elems<T>();
     const int lane = threadIdx.x & 31;
@@ -492,15 +491,17 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, int sta
         }
         if (lane == 0) {
             sm.item[slot] = t;
-            sm.held = nullptr;
+            if constexpr (QUEUE) sm.held = nullptr;
         }
         __syncwarp();
-        if (lane == 0 && stall != (int)i + 1) arrive(&sm.it_full[slot]);
+        if (lane == 0) arrive(&sm.it_full[slot]);
         return true;
     };
     auto take = [&](Item& t, Source& from) {
         next(t, from);
-        if (lane == 0 && t.K) sm.held = t.sd;
+        if constexpr (QUEUE) {
+            if (lane == 0 && t.K) sm.held = t.sd;
+        }
     };
     bool ok = true;
     unsigned int i = 0;
@@ -889,8 +890,15 @@ __device__ __forceinline__ void retire_tile(const SM& sm, const Item& it, int sl
     }
 }
 
-// After run_roles, by one thread of a CTA that gave up: flags the sessions of every tile that it took
-// and whose sums it did not record, which are those in the slots and the one in the manager's hands.
+// QUEUE, before run_roles, by one thread: no tile in the second slot (the first gets one before any wait)
+// and none in the manager's hands.
+template <typename SM>
+__device__ __forceinline__ void none_taken(SM& sm) {
+    sm.item[1].K = 0;
+    sm.held = nullptr;
+}
+// QUEUE, after run_roles, by one thread of a CTA that gave up: flags the sessions of every tile that it
+// took and whose sums it did not record, which are those in the slots and the one in the manager's hands.
 template <typename SM>
 __device__ __forceinline__ void flag_failed(const SM& sm) {
     for (int k = 0; k < 2; ++k)
@@ -898,11 +906,11 @@ __device__ __forceinline__ void flag_failed(const SM& sm) {
     if (sm.held) atomicOr(&sm.held->status, LOC_DEV_ERR_TIMEOUT);
 }
 
-// The roles of the CTA's warps; next, done and stall as for manage().  next() gives a tile's geometry and
-// input(item, src) what earlier work on the stream wrote (scale, restart flag); for the first tile
-// begin() runs between them, the barriers, the plan and the map mask being set up by then: the
-// manager's planes travel while the other warps read the map.
-template <typename T, bool AM, bool RAG, typename Next, typename Begin, typename Input, typename Done>
+// The roles of the CTA's warps; next and done as for manage(), stall as for init_barriers().  next()
+// gives a tile's geometry and input(item, src) what earlier work on the stream wrote (scale, restart
+// flag); for the first tile begin() runs between them, the barriers, the plan and the map mask being
+// set up by then: the manager's planes travel while the other warps read the map.
+template <typename T, bool AM, bool RAG, bool QUEUE, typename Next, typename Begin, typename Input, typename Done>
 __device__ __forceinline__ void run_roles(Smem<T>& sm, int stall, Next next, Begin begin, Input input, Done done) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Item it{};
@@ -910,7 +918,7 @@ __device__ __forceinline__ void run_roles(Smem<T>& sm, int stall, Next next, Beg
     if (warp == NO) {
         next(it, src);
         if (lane == 0) {
-            init_barriers(sm);
+            init_barriers(sm, stall);
             sm.item[0] = it;
         }
         fill_plan<RAG>(sm, 0, it, src, lane);
@@ -926,14 +934,14 @@ __device__ __forceinline__ void run_roles(Smem<T>& sm, int stall, Next next, Beg
         if (lane == 0) {
             sm.item[0].in_scale = it.in_scale;
             sm.item[0].reinit = it.reinit;
-            if (stall != 1) arrive(&sm.it_full[0]);
+            arrive(&sm.it_full[0]);
         }
         __syncwarp();
     }
     if (warp < NO + 1) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsOut));
         if (warp < NO) output<T, AM, RAG>(sm, threadIdx.x);
-        else manage<T, RAG>(sm, it, src, stall, [&](Item& t, Source& s) {
+        else manage<T, RAG, QUEUE>(sm, it, src, [&](Item& t, Source& s) {
             next(t, s);
             input(t, s);
         }, done);

@@ -95,18 +95,19 @@ def test_a_batch_that_gives_up_at_its_first_tile(use_graph):
 
 
 def test_a_batch_session_that_was_finished_stays_usable():
-    """Every CTA's fourth tile is withheld.  The first session's tiles (longest bins, so taken first,
-    one for every second SM) were recorded by then and it is not failed; the second one's were not."""
+    """Every CTA's second tile is withheld.  The first session's tiles (the longest bins, so taken first, by
+    eight CTAs) are first ones: they are recorded when a third tile is taken, and the session goes on.  The
+    second session has six tiles a CTA and fails."""
     import torch
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    first, second = (28, 64 * (n_sm // 2), 12), (28 * 8, 64 * n_sm, 8)
+    first, second = (28, 64 * 8, 12), (28 * 6, 64 * n_sm, 8)
     want = beliefs_after(2, *first, tile=3)
     hs = [session(*first), session(*second, seed=1)]
     b = loc.loc_batch_create(hs, tile=3)
     try:
         loc.loc_batch_step(b, 0.03, 0.01, 0.02)
         loc.loc_batch_sync(b)
-        loc.loc_debug_step_stall(4)
+        loc.loc_debug_step_stall(2)
         loc.loc_batch_step(b, 0.03, 0.01, 0.02)
         with pytest.raises(loc.LocError) as e:
             loc.loc_batch_sync(b)
@@ -123,6 +124,7 @@ def test_a_batch_session_that_was_finished_stays_usable():
 
 
 def test_hook_arguments():
-    with pytest.raises(loc.LocError) as e:
-        loc.loc_debug_step_stall(-1)
-    assert e.value.status == loc.LOC_ERR_INVALID_ARG
+    for bad in (-1, 3):
+        with pytest.raises(loc.LocError) as e:
+            loc.loc_debug_step_stall(bad)
+        assert e.value.status == loc.LOC_ERR_INVALID_ARG
