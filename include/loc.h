@@ -109,9 +109,10 @@ typedef struct {
                                   With tile = 0 a grid of at least 8 sixteen-row tiles per SM
                                   takes 17 (FP32) or 3 (16-bit storage), smaller grids 16. */
 
-/* Propagation kernel selection: AUTO takes the TMA-tiled kernel when it applies (x/y radius
- * 2, theta radius 3, K >= 8, W a multiple of 16 bytes of storage) and the generic one
- * otherwise; forcing TILED where it does not apply fails loc_create with INVALID_ARG. */
+/* Propagation kernel selection.  With x/y radius 2, theta radius 3 and K >= 8, AUTO takes the
+ * TMA-tiled kernel where rows are a multiple of 16 bytes of storage (loc_params.tile picks its
+ * configuration) and the streaming kernel without TMA on other widths; the generic kernel
+ * otherwise.  Forcing TILED where it does not apply fails loc_create with INVALID_ARG. */
 enum { LOC_KERNEL_AUTO = 0, LOC_KERNEL_GENERIC = 1, LOC_KERNEL_TILED = 2 };
 
 /* Fill *p with the defaults: sigma_xy 0.5 cells, sigma_theta 1 bin, radii ceil(3 sigma),
@@ -212,7 +213,7 @@ loc_status loc_estimate(loc_handle h, double radius_m, int dk, loc_estimate_t* o
  *                 map, Section III-A.3), LOC_MAP_SUM = sum over channels (marginal).
  *   loc_argmax:   the most probable state (k, j, i) and its probability; ties go to the
  *                 lowest linear index in [K][H][W] order.  After a loc_step through a
- *                 warp-specialised tile configuration (6, 7, 13-16) the step kernel has
+ *                 tile configuration that fuses it (6, 7, 13-16) the step kernel has
  *                 already combined this argmax, and the call only reads it back; otherwise
  *                 it makes one pass over the tensor. */
 loc_status loc_belief(loc_handle h, float* out, size_t n);

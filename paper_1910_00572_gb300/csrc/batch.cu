@@ -1,11 +1,11 @@
 // Batched propagation: many sessions of uneven H x W x K stepped by one persistent launch.
 //
-// The grid is sized to the GPU (resident CTAs per SM x SMs).  Each CTA repeatedly takes the
-// next (session, tile) item from a device work queue and runs Algorithm 1's propagation on that
-// session's tile (the streaming tiles of stream.cuh, or the synchronous run_tile); the CTA that finishes a session's last
-// tile combines the session's FP64 tile partials into its normaliser Z (Eq. 9) in the same
-// fixed order as a single-session launch, so a session's result does not depend on which
-// other sessions share the launch.
+// The grid is sized to the GPU (resident CTAs per SM x SMs; one per SM for the streaming tiles).
+// Each CTA repeatedly takes the next (session, tile) item from a device work queue and runs
+// Algorithm 1's propagation on that session's tile (the streaming tiles of stream.cuh, or the
+// synchronous run_tile); the CTA that finishes a session's last tile combines the session's FP64
+// tile partials into its normaliser Z (Eq. 9) in the same fixed order as a single-session launch,
+// so a session's result does not depend on which other sessions share the launch.
 #include "kernels.h"
 #include "stream.cuh"
 

@@ -422,7 +422,7 @@ LOC_API loc_status loc_step(loc_handle h, double u, double v, double w) {
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
     step_done(h);
-    // the warp-specialised tiled kernels write the argmax of the new tensor
+    // some tile configurations write the argmax of the new tensor
     h->am_valid = !h->aniso && h->tiled && step_tiled_fuses_argmax(h->tile_cfg);
     return LOC_OK;
 }

@@ -21,12 +21,14 @@
 // shared memory with two CTA barriers a plane: 42 to 53 thread instructions a cell and issue
 // 41 to 52 % busy.  Here a cell costs 35 (FP32) to 39 (BF16), eight
 // planes are in the works at once, and the latency of one plane's chain no longer counts.
-// Every value is computed with the operations and the order of the passes in tiled_common.cuh,
-// and a thread of the output warps sums the same cells, so tensors and normalisers are those
-// of the 128-thread synchronous configuration bit for bit.  Before and after, us a step: 64 x 64 x
-// 16 FP32 27.3 -> 16.7, 500 x 500 x 128 111 -> 64, 512 x 512 x 64 63.5 -> 39.7, 1816 x 1816 x 36 FP16
-// 310 -> 253, 2048 x 2048 x 72 BF16 725 -> 550 (2.2 TB/s) and FP32 793 -> 543 (4.5 TB/s).  What bounds
-// it now: the output warps' instruction issue and latency, two of them on a scheduler.
+// Every value is computed with the operations and the order of the passes in tiled_common.cuh, so
+// tensors are those of the other tile configurations bit for bit.  A thread of the output warps sums
+// its four rows before each compensated addition of the normaliser, as the synchronous configurations
+// with four rows a thread do (two by two on ragged rows, as the generic kernel does).  Before and
+// after, us a step: 64 x 64 x 16 FP32 27.3 -> 16.6, 500 x 500 x 128 111 -> 63, 512 x 512 x 64 63.5 -> 39.7,
+// 1816 x 1816 x 36 FP16 310 -> 249, 2048 x 2048 x 72 BF16 725 -> 552 (2.2 TB/s) and FP32 793 -> 543 (4.5
+// TB/s).  What bounds it now: the output warps' instruction issue and latency, two of them on a
+// scheduler.
 #pragma once
 #include <type_traits>
 
@@ -389,7 +391,8 @@ __device__ __forceinline__ void init_barriers(Smem<T>& sm, int stall) {
 }
 
 // The map mask over item t's halo region, by threads k of n.  The grid's width is a multiple of
-// 4 cells, so the map comes in whole words; W words a thread are in flight at once.
+// 4 cells (and device buffers are aligned to 16 bytes), so the map comes in whole words; W words a
+// thread are in flight at once.
 constexpr int MWORDS = 19;             // words a row: columns -4 .. 71 of the tile
 template <int N, bool RAG, typename SM>
 __device__ __forceinline__ void fill_mask(SM& sm, int slot, const Item& t, int k) {
