@@ -158,7 +158,7 @@ batch_stream_kernel(const BatchStatic* __restrict__ ss, const BatchTick* __restr
             const int cur = tk[sess].cur;
             const BatchStatic& S = ss[sess];
             // a dry run times the steady state (TMA input) whatever the session's restart flag
-            src.reinit = dry ? 0 : S.sd->reinit;
+            it.reinit = src.reinit = dry ? 0 : S.sd->reinit;
             src.sh = shifts + S.sh_off;
             src.tmap = reinterpret_cast<const CUtensorMap*>(S.tmap[cur]);
             // the tensor map lives in global memory, written by a copy before the launch

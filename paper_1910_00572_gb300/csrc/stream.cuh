@@ -65,8 +65,8 @@ struct OCfg {                          // rows of an output thread (2 columns ea
 // One tile of work, as the manager hands it to the other warps.  K = 0: no more tiles.
 struct Item {
     void* out;
-    const void* in;                    // ragged rows only: X_{t-1} ...
-    int reinit;                        // ... or M in its place
+    const void* in;                    // ragged rows only: X_{t-1}
+    int reinit;                        // M is read in the place of X_{t-1}
     const uint8_t* trav;
     const float* corr;
     int K, H, W, ty0, tx0;
@@ -364,11 +364,43 @@ __device__ __forceinline__ int load_rows(T* raw, const Item& it, int p, int x, i
     return xo;
 }
 
+// A restart's input in place of a plane's TMA box, by its blur warp: the map (0 / 1) at columns x (a
+// multiple of a 16-byte chunk) and rows y0 .. .  The grid's width is a multiple of 4 cells here, so a
+// word of the map lies in the grid or outside it as a whole; four words a lane are in flight.  (With
+// the manager warp filling every plane's box a cell at a time, a restart's step took 3.7 ms instead of
+// 0.55 at 2048 x 2048 x 72 BF16; 0.69 like this.)
+template <typename T>
+__device__ __forceinline__ void load_map(T* raw, const Item& it, int x, int y0) {
+    const int lane = threadIdx.x & 31, H = it.H, W = it.W;
+    constexpr int BWT = box_w<T>(), WORDS = BWT / 4, ALL = RAW_H * WORDS;
+    static_assert(BWT % 4 == 0, "whole words a row");
+#pragma unroll 1
+    for (int q0 = lane; q0 < ALL; q0 += 4 * 32) {
+        uint32_t m[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const int q = q0 + 32 * n, gy = y0 + q / WORDS, gx = x + 4 * (q % WORDS);
+            m[n] = q < ALL && gy >= 0 && gy < H && gx >= 0 && gx < W
+                       ? *reinterpret_cast<const uint32_t*>(it.trav + (size_t)gy * W + gx) : 0u;
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const int q = q0 + 32 * n;
+            struct alignas(4 * sizeof(T)) Four {
+                T v[4];
+            } o;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) o.v[b] = T((float)((m[n] >> (8 * b)) & 0xFFu));
+            if (q < ALL) *reinterpret_cast<Four*>(raw + 4 * q) = o;
+        }
+    }
+}
+
 // The manager's private side of a tile: where its planes come from.
 struct Source {
     const CUtensorMap* tmap;
     const Shift* sh;
-    int reinit;                        // read the input as M (uniform restart) instead of TMA
+    int reinit;                        // the input is M (uniform restart): no TMA, the blur warps read it
 };
 
 // stall: the CTA's first (1) or second (2) tile is never handed over, since its barrier waits for one
@@ -460,19 +492,13 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
         if (g >= NB && !wait(sm, &sm.raw_empty[s], ((g / NB) - 1) & 1)) return false;
         const int4 pl = plan[p];
         const int x_al = pl.x & ~(AL - 1), y0 = pl.y;
-        if (src.reinit) {
-            // the uniform input, written where TMA would have put the box (M as 0/1)
-            for (int q = lane; q < RAW_H * box_w<T>(); q += 32) {
-                const int gy = y0 + q / box_w<T>(), gx = x_al + q % box_w<T>();
-                float v = 0.0f;
-                if (gy >= 0 && gy < it.H && gx >= 0 && gx < it.W) v = (float)it.trav[(size_t)gy * it.W + gx];
-                sm.raw[s][q] = T(v);
+        if (lane == 0) {
+            if (src.reinit) {          // the stage is the blur warp's, to fill with the map
+                arrive(&sm.raw_full[s]);
+            } else {
+                bar_expect(&sm.raw_full[s], kBoxBytes);
+                tma_load(&sm.raw[s][0], src.tmap, &sm.raw_full[s], x_al, y0, p);
             }
-            __syncwarp();
-            if (lane == 0) arrive(&sm.raw_full[s]);
-        } else if (lane == 0) {
-            bar_expect(&sm.raw_full[s], kBoxBytes);
-            tma_load(&sm.raw[s][0], src.tmap, &sm.raw_full[s], x_al, y0, p);
         }
         ++g;
         return true;
@@ -521,8 +547,6 @@ __device__ __forceinline__ void manage(Smem<T>& sm, Item it, Source src, Next ne
                 ok = publish(i + 1, nit, nsrc);
             }
         }
-        // raw stages that plain stores wrote (a restart's planes) may take TMA copies next
-        if (src.reinit) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         it = nit;
         src = nsrc;
         plan = sm.plan[(i + 1) & 1];
@@ -544,6 +568,7 @@ __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
         const Item& it = sm.item[slot];
         const unsigned int K = it.K;
         if (K == 0) return;
+        const bool restart = !RAG && it.reinit;
         const f2 g0 = pk(it.g0, it.g0), g1 = pk(it.g1, it.g1), g2 = pk(it.g2, it.g2);
         for (; g < base + K; g += NB) {
             const uint32_t ph = (g / NB) & 1;
@@ -551,6 +576,13 @@ __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
             int xo;
             if constexpr (RAG) xo = load_rows<T>(sm.raw[w], it, channel<true>(g - base, K), pl.x, pl.y);
             else xo = pl.x & (align_elems<T>() - 1);
+            if constexpr (!RAG) {
+                if (restart) {
+                    if (!wait(sm, &sm.raw_full[w], ph)) return;
+                    load_map<T>(sm.raw[w], it, pl.x - xo, pl.y);
+                    __syncwarp();
+                }
+            }
             if (g >= NB && !wait(sm, &sm.x_empty[w], ph ^ 1)) return;
             if constexpr (RAG) {
                 asm volatile("cp.async.wait_all;" ::: "memory");
@@ -560,6 +592,8 @@ __device__ __forceinline__ void blur(Smem<T>& sm, int w) {
             }
             blur_any<T, RAG>(sm.raw[w], &sm.mk[slot][0][0], &sm.X[w][0][0], xo, __int_as_float(pl.z),
                              __int_as_float(pl.w), g0, g1, g2);
+            // the stage that plain stores wrote may take a TMA copy next
+            if (restart) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
                 if constexpr (!RAG) arrive(&sm.raw_empty[w]);
