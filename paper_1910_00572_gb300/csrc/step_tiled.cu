@@ -513,11 +513,14 @@ int step_tiled_default_cfg(int H, int W, int K, int storage) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         nsm = 152;
-    // The streaming kernel on every grid (64 x 64 x 16 to 2048 x 2048 x 72: 0.64 to 0.79 of the
-    // time of the tile configurations it took the place of).  The argmax is combined in the step
-    // (16) where a pose is likely to be read after every step and the step is short: it costs
-    // 4 us at 512 x 512 x 64 (43 against 39), the pass it saves 17; on grids of at least 8
-    // sixteen-row tiles per SM it is left to the pass (17 for FP32, 3 for 16-bit storage).
+    // The streaming kernel on every grid (64 x 64 x 16 to 2048 x 2048 x 72: 0.57 to 0.81 of the
+    // time of the tile configurations it took the place of).  What is left to choose is whether the
+    // step combines the argmax (16) or leaves it to loc_argmax's pass (3 and 17, one kernel).  Back to
+    // back, us: 512 x 512 x 64 FP32 a step takes 38.5 with it and 35.9 without, a step and loc_argmax
+    // 56 and 70; 1024 x 1024 x 36 96 / 85 and 117 / 144; 2048 x 2048 x 72 BF16 600 / 546 and 620 / 711.
+    // So each is right for one way of use at every size.  Small maps, where the pass and its launch
+    // weigh most, combine it; from 8 x 16 x 64 x (SMs) cells on (1.25 million here) a step alone comes
+    // first.  The line is where it was for the configurations before.
     const long long cols = (W + TW - 1) / TW;
     if (cols * ((H + 15) / 16) >= 8LL * nsm) return storage == LOC_F32 ? 17 : 3;
     return 16;

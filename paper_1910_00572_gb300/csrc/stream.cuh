@@ -25,8 +25,8 @@
 // tensors are those of the other tile configurations bit for bit.  A thread of the output warps sums
 // its four rows before each compensated addition of the normaliser, as the synchronous configurations
 // with four rows a thread do (two by two on ragged rows, as the generic kernel does).  Before and
-// after, us a step: 64 x 64 x 16 FP32 27.3 -> 16.6, 500 x 500 x 128 111 -> 63, 512 x 512 x 64 63.5 -> 39.7,
-// 1816 x 1816 x 36 FP16 310 -> 249, 2048 x 2048 x 72 BF16 725 -> 552 (2.2 TB/s) and FP32 793 -> 543 (4.5
+// after, us a step: 64 x 64 x 16 FP32 27.3 -> 16.4, 500 x 500 x 128 111 -> 63, 512 x 512 x 64 63.5 -> 39.5,
+// 1816 x 1816 x 36 FP16 310 -> 250, 2048 x 2048 x 72 BF16 725 -> 548 (2.2 TB/s) and FP32 793 -> 542 (4.5
 // TB/s).  What bounds it now: the output warps' instruction issue and latency, two of them on a
 // scheduler.
 #pragma once
